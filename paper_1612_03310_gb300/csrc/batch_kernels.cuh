@@ -11,10 +11,8 @@
 // Work lists: the flat phases number their blocks member after member, and
 // a block finds its member by binary search in the table's prefix of block
 // counts (blk[phase][m] .. blk[phase][m+1]); the particle step is persistent
-// (one CTA set for the device) and walks the members' dense tile lists in
-// turn, each CTA starting at its own member, taking tiles from a member's
-// counter until that member is done, then the sparse lists, then the lost
-// tails.
+// (one CTA set for the device) and takes every member's units from one
+// counter, then the lost tails; the sparse tiles have a launch of their own.
 #pragma once
 #include "common.cuh"
 #include "field_kernels.cuh"
@@ -146,30 +144,33 @@ __global__ void __launch_bounds__(256) kb_power(const BatchMember<T, U>* __restr
 }
 
 // The particle step of every member is k_push_tiled<.., kBatch = true>
-// (tile_push.cuh): persistent CTAs take every member's non-empty tiles from
-// one counter; kb_tile_prefix numbers those tiles member after member (from
-// the tile counts the last re-sort left) and clears the counter.
+// (tile_push.cuh): persistent CTAs take every member's units from one
+// counter (k_push_sparse strides over their sparse tiles); kb_tile_prefix
+// numbers both member after member (from the lists the last re-sort left)
+// and clears the counter.
 template <typename T, typename U>
 __global__ void __launch_bounds__(1024) kb_tile_prefix(const BatchMember<T, U>* __restrict__ mem,
                                                        int M, int* __restrict__ pref,
+                                                       int* __restrict__ spref,
                                                        int* __restrict__ work) {
-  __shared__ int ws[32];
-  int base = 0;
+  __shared__ Pair ws[32];
+  Pair base = 0;
   for (int c0 = 0; c0 < M; c0 += blockDim.x) {
     const int m = c0 + threadIdx.x;
-    int n = 0;
+    Pair n = 0;
+    if (m < M) n = pair_of(mem[m].units[0].x, mem[m].st->n_sparse);
+    Pair tot;
+    const Pair ex = base + block_exclusive_scan(n, ws, &tot);
     if (m < M) {
-      const StepState* st = mem[m].st;
-      n = st->n_tiles + st->n_sparse;
+      pref[m] = pair_lo(ex);
+      spref[m] = pair_hi(ex);
     }
-    int tot;
-    const int ex = block_exclusive_scan(n, ws, &tot);
-    if (m < M) pref[m] = base + ex;
     base += tot;
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    pref[M] = base;
+    pref[M] = pair_lo(base);
+    spref[M] = pair_hi(base);
     *work = 0;
   }
 }
@@ -181,7 +182,8 @@ __global__ void __launch_bounds__(kScanBlock) kb_scan_partials(
   const int g = blockIdx.x;
   const int mi = member_of(blk, M, g);
   const BatchMember<T, U>& m = mem[mi];
-  scan_partials_body(m.count, m.nkeys, m.sparse_below, m.scan_part, g - blk[mi]);
+  scan_partials_body(m.count, m.offset, m.nkeys, m.sparse_below, m.chunk, m.scan_part,
+                     g - blk[mi]);
 }
 
 // Second pass (advances every member's step counter).
@@ -191,8 +193,8 @@ __global__ void __launch_bounds__(kScanBlock) kb_scan_final(
   const int g = blockIdx.x;
   const int mi = member_of(blk, M, g);
   const BatchMember<T, U>& m = mem[mi];
-  scan_final_body(m.count, m.offset, m.tiles, m.nkeys, m.sparse_below, m.scan_part, m.scan_nb,
-                  m.st, 1, g - blk[mi]);
+  scan_final_body(m.count, m.offset, m.tiles, m.units, m.nkeys, m.sparse_below, m.chunk,
+                  m.scan_part, m.scan_nb, m.st, 1, g - blk[mi]);
 }
 
 // The re-sort's slot map (slot_one), 256 particles per block.

@@ -22,6 +22,7 @@ struct PushArgs {
   const int* perm;    // slot of the tile order -> position in P
   const int* offset;
   const int* tiles;
+  const int4* units;  // work units (k_scan_final)
   int* count;
   int* key;
   int* rank;
@@ -49,6 +50,7 @@ struct BatchMember {
   int* perm;         // slot of the tile order -> position in A (the re-sort's output)
   int* offset;
   int* tiles;
+  int4* units;
   int* count;
   int* key;
   int* rank;
@@ -63,6 +65,7 @@ struct BatchMember {
   int nkeys;
   int scan_nb;
   int sparse_below;
+  int chunk;
   int fused_mur;  // first-order Mur at the x faces inside the z-marching loop
   unsigned char* dirty;  // source-tile flags, as in PushArgs
   int dirty_words;

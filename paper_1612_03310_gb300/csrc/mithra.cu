@@ -68,6 +68,7 @@ struct mithra_sim {
   int* count = nullptr;
   int* offset = nullptr;
   int* tiles = nullptr;  // non-empty tile list written by the scan
+  int4* units = nullptr;  // the particle step's work units, written by the scan
   // source-tile flags of the two level parities (StencilP::dirty), each
   // dirty_words words
   unsigned char* dirty = nullptr;
@@ -137,6 +138,8 @@ struct mithra_sim {
 };
 
 void batch_mark_dirty(mithra_batch* b);  // defined with the batch
+// particles of all members of a batch
+void batch_totals(const mithra_batch* b, int64_t* particles);
 
 namespace {
 
@@ -402,16 +405,59 @@ Parts<T, U> parts_of(mithra_sim* s, int b) {
   return P;
 }
 
+// Most slots of a particle-step unit (a multiple of its 256 threads) for np
+// particles, of one simulation or of a whole batch, on `ctas` persistent
+// CTAs: a third of an even share, so that no tile's work outlasts the rest
+// (262144 particles in 64 x 64 x 256 cells, 3000 in a heavy tile: particle
+// step 96 us with one CTA a tile, 43 us split; a sixth of the share was
+// slower again, each unit staging its tile's fields anew).
+int unit_chunk(int64_t np, int ctas) {
+  const int64_t c = (np / (3 * (int64_t)ctas) + kMinChunk - 1) / kMinChunk * kMinChunk;
+  return (int)std::min<int64_t>(std::max<int64_t>(c, kMinChunk), 16384);
+}
+
+// Entries of the unit list: its header, every tile, and the further units of
+// the tiles that are split.
+int64_t unit_entries(int64_t np, int64_t nkeys) { return 1 + nkeys + np / kMinChunk; }
+
+// Particles that share the device with this simulation's: its batch's, or its
+// own.
+int64_t particles_beside(const mithra_sim* s) {
+  int64_t np = s->np;
+  if (s->in_batch) batch_totals(s->in_batch, &np);
+  return np;
+}
+
+// Tiles below this many particles take the sparse path (0: none): the
+// caller's threshold, or 32 (FP64: 64) on grids of many tiles per CTA, where
+// the staged path's time is its number of tiles (128 x 128 x 1024 cells, 2^21
+// particles, P32_U64: 252 us at 0, 240 at 16 to 32, 273 at 64; FP64 on 96 x 80
+// x 384 cells, 4e5 particles: 536, 471 at 32, 458 at 64).  With few tiles a
+// CTA the lone warp of a sparse tile takes longer than a CTA with it.
+int sparse_below(const mithra_sim* s) {
+  if (s->push_variant != 1 || !s->have_tm) return 0;
+  if (s->push_sparse_below > 0) return s->push_sparse_below;
+  if (s->nkeys < 16 * s->push_grid) return 0;
+  return s->prec == MITHRA_P64 ? 64 : 32;
+}
+
+// Blocks of the sparse tiles' kernel: eight a multiprocessor (32 warps), so
+// that the device takes some 5000 sparse tiles at once.
+unsigned sparse_grid(int n_sm) { return 8u * n_sm; }
+
 // Two-pass scan of the per-tile counts (see k_scan_final), on stream q
 // (default: the simulation's).
+template <bool kRestored = false>
 void launch_scan(mithra_sim* s, int advance, cudaStream_t q = nullptr) {
   if (!q) q = s->stream;
   const int nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
-  const int sparse_below = s->push_variant == 1 ? s->push_sparse_below : 0;
-  k_scan_partials<<<nb, kScanBlock, 0, q>>>(s->count, s->nkeys, sparse_below, s->scan_part);
-  k_scan_final<<<nb, kScanBlock, 0, q>>>(s->count, s->offset, s->tiles, s->nkeys,
-                                                 sparse_below, s->scan_part, nb, s->dstate,
-                                                 advance);
+  const int below = sparse_below(s);
+  const int chunk = unit_chunk(particles_beside(s), s->push_grid);
+  k_scan_partials<kRestored><<<nb, kScanBlock, 0, q>>>(s->count, s->offset, s->nkeys,
+                                                       below, chunk, s->scan_part);
+  k_scan_final<kRestored><<<nb, kScanBlock, 0, q>>>(s->count, s->offset, s->tiles, s->units,
+                                                    s->nkeys, below, chunk, s->scan_part,
+                                                    nb, s->dstate, advance);
 }
 
 // Instantiated forms of the particle step: without lo parts (P32, P64) and
@@ -565,16 +611,17 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
     else
       k_mur_boundary<false, T><<<mg, dim3(32, 8), 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S);
     if (s->stencil_variant == 2) {
+      const int lz = s->lz;
       dim3 blk(32, 8, 1);
-      dim3 grd((s->g.nx + 31) / 32, (s->g.ny + 7) / 8, (s->g.nz + s->lz - 1) / s->lz);
+      dim3 grd((s->g.nx + 31) / 32, (s->g.ny + 7) / 8, (s->g.nz + lz - 1) / lz);
       if (L0 && fused)
-        k_potential_zloop_mur1<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, s->lz);
+        k_potential_zloop_mur1<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else if (L0)
-        k_potential_zloop<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, s->lz);
+        k_potential_zloop<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else if (fused)
-        k_potential_zloop_mur1<false, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, s->lz);
+        k_potential_zloop_mur1<false, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else
-        k_potential_zloop<false, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, s->lz);
+        k_potential_zloop<false, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
     } else if (s->stencil_variant == 1 && s->have_tm && !L0) {
       dim3 grd((s->g.nx + kMX - 1) / kMX, (s->g.ny + kMY - 1) / kMY,
                (s->g.nz + s->lz - 1) / s->lz);
@@ -607,8 +654,11 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         k_seed_tfsf<false, T><<<grd, blk, 0, s->stream>>>(sp, s->seed, s->dstate, P1, L1, Dn);
     }
   }
-  // with per-kernel timing every kernel stays on the simulation's stream
-  const bool branch = !s->profiling && (s->power_cap > 0 || s->spec_nf > 0);
+  // the sparse tiles' kernel and the plane diagnostics run beside the tiled
+  // particle step; with per-kernel timing every kernel stays on the
+  // simulation's stream
+  const bool sparse = s->np > 0 && s->push_variant == 1 && s->have_tm && sparse_below(s) > 0;
+  const bool branch = !s->profiling && (s->power_cap > 0 || s->spec_nf > 0 || sparse);
   cudaStream_t dq = s->stream;
   if (branch) {
     cudaEventRecord(s->ev_fork, s->stream);
@@ -640,10 +690,17 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
       constexpr bool kAnyLo = !push_form_plain<T, U>();  // a form that exists, for the type
       if (s->push_variant == 1 && s->have_tm) {
         decltype(&k_push_tiled<false, T, U, kAnyLo>) kern = nullptr;
+        decltype(&k_push_sparse<false, T, U, kAnyLo>) kern_sp = nullptr;
         if constexpr (push_form_plain<T, U>())
-          if (!lo) kern = opt ? k_push_tiled<true, T, U> : k_push_tiled<false, T, U>;
+          if (!lo) {
+            kern = opt ? k_push_tiled<true, T, U> : k_push_tiled<false, T, U>;
+            kern_sp = opt ? k_push_sparse<true, T, U> : k_push_sparse<false, T, U>;
+          }
         if constexpr (push_form_lo<T, U>())
-          if (lo) kern = opt ? k_push_tiled<true, T, U, true> : k_push_tiled<false, T, U, true>;
+          if (lo) {
+            kern = opt ? k_push_tiled<true, T, U, true> : k_push_tiled<false, T, U, true>;
+            kern_sp = opt ? k_push_sparse<true, T, U, true> : k_push_sparse<false, T, U, true>;
+          }
         if (!kern) return fail(s, MITHRA_EINVAL, "no particle-step form for this precision");
         PushParams<T, U, false> prm;
         prm.tm_pn = s->tm_box[1 - s->cur];
@@ -659,6 +716,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         pa.perm = s->perm;
         pa.offset = s->offset;
         pa.tiles = s->tiles;
+        pa.units = s->units;
         pa.count = s->count;
         pa.key = s->key;
         pa.rank = s->rank;
@@ -667,6 +725,8 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         pa.dirty = s->dirty;
         pa.dirty_words = s->dirty_words;
         pa.cur = s->cur;
+        if (sparse)
+          kern_sp<<<sparse_grid(s->n_sm), kSparseThreads, 0, branch ? s->side : s->stream>>>(prm);
         // a programmatic dependent launch: the grid is scheduled as the
         // work before it drains and waits at its start for that work
         cudaLaunchConfig_t cfg = {};
@@ -929,7 +989,7 @@ void lab_of(const mithra_sim* s, int32_t kp, double t, double* t_lab, double* z_
 void free_all(mithra_sim* s) {
   if (s->stream) cudaStreamSynchronize(s->stream);
   void* ptrs[] = {s->P[0], s->P[1], s->PL[0], s->PL[1], s->D, s->S, s->pbuf[0], s->pbuf[1], s->perm, s->key, s->rank, s->count,
-                  s->offset, s->tiles, s->dirty, s->scan_part, s->dstate, s->d_scalar, s->d_power_rec,
+                  s->offset, s->tiles, s->units, s->dirty, s->scan_part, s->dstate, s->d_scalar, s->d_power_rec,
                   s->d_spec_omega, s->d_spec_acc, s->d_spec_out, s->d_spec_samples,
                   s->d_bunch_rec, s->d_bunch_part};
   for (void* p : ptrs)
@@ -982,6 +1042,7 @@ mithra_status mithra_footprint(const mithra_grid* grid, int64_t n_particles,
   b += 2 * (int64_t)particle_buffer_bytes(n_particles, precision);
   b += 3 * n_particles * (int64_t)sizeof(int);                   // slot map, key, rank
   b += 3 * (nkeys + 2) * (int64_t)sizeof(int);                   // count, offset, tiles
+  b += unit_entries(n_particles, nkeys) * (int64_t)sizeof(int4);  // particle-step units
   b += 8 * ((nkeys + 3) / 4);                                     // source-tile flags
   b += (nkeys / kScanBlock + 2) * (int64_t)sizeof(int4);         // scan block sums
   b += (int64_t)sizeof(StepState) + (int64_t)sizeof(double);
@@ -1070,6 +1131,7 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
             dalloc((void**)&s->count, sizeof(int) * (size_t)(s->nkeys + 2)) &&
             dalloc((void**)&s->offset, sizeof(int) * (size_t)(s->nkeys + 2)) &&
             dalloc((void**)&s->tiles, sizeof(int) * (size_t)(s->nkeys + 1)) &&
+            dalloc((void**)&s->units, sizeof(int4) * (size_t)unit_entries(np, s->nkeys)) &&
             dalloc((void**)&s->dirty, 8 * (size_t)s->dirty_words) &&
             dalloc((void**)&s->scan_part, sizeof(int4) * (size_t)(s->nkeys / kScanBlock + 2)) &&
             dalloc((void**)&s->dstate, sizeof(StepState)) &&
@@ -1738,6 +1800,8 @@ mithra_status mithra_restore(mithra_sim* s, const void* in) {
     MCHECK(s, cudaMemcpyAsync(part.dev, p, part.bytes, cudaMemcpyHostToDevice, s->stream));
     p += part.bytes;
   }
+  // the tile and unit lists for this simulation's own launch choices
+  if (s->np > 0) launch_scan<true>(s, 0);
   mark_sources_everywhere(s);
   MCHECK(s, refresh_mirror(s));
   mithra_status st = sync_status(s);
@@ -1805,7 +1869,7 @@ struct mithra_batch {
   size_t table_bytes = 0;
   int* d_blk = nullptr;     // block prefixes, kBPCount x (M + 1)
   size_t blk_bytes = 0;
-  int* d_pref = nullptr;    // the particle step's tile prefix (M + 1) and counter
+  int* d_pref = nullptr;    // the particle step's unit and sparse-tile prefixes, unit counters
   size_t pref_bytes = 0;
   int* d_zblk = nullptr;    // boundary and update block prefixes, per group from 0
   size_t zblk_bytes = 0;
@@ -1817,6 +1881,11 @@ struct mithra_batch {
 
 void batch_mark_dirty(mithra_batch* b) {
   if (b) b->dirty = true;
+}
+
+void batch_totals(const mithra_batch* b, int64_t* particles) {
+  *particles = 0;
+  for (const mithra_sim* s : b->sims) *particles += s->np;
 }
 
 namespace {
@@ -1895,6 +1964,7 @@ BatchMember<T, U> member_entry(mithra_sim* s, int c, int pb) {
   m.perm = s->perm;
   m.offset = s->offset;
   m.tiles = s->tiles;
+  m.units = s->units;
   m.count = s->count;
   m.key = s->key;
   m.rank = s->rank;
@@ -1909,7 +1979,8 @@ BatchMember<T, U> member_entry(mithra_sim* s, int c, int pb) {
   m.power_plane = s->power_plane;
   m.nkeys = s->nkeys;
   m.scan_nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
-  m.sparse_below = 0;  // the fused particle step stages every tile
+  m.sparse_below = sparse_below(s);
+  m.chunk = unit_chunk(particles_beside(s), s->push_grid);
   m.fused_mur = s->g.boundary == 1;
   set_source_flags(s, c, &m.sp);
   m.dirty = s->dirty;
@@ -1932,6 +2003,7 @@ PushArgs<T, U> push_args_of(const BatchMember<T, U>& m) {
   a.perm = m.perm;
   a.offset = m.offset;
   a.tiles = m.tiles;
+  a.units = m.units;
   a.count = m.count;
   a.key = m.key;
   a.rank = m.rank;
@@ -1961,7 +2033,8 @@ mithra_status capture_fused_typed(mithra_batch* b) {
     const mithra_grid& g = s->g;
     const long long nb[kBPCount] = {
         (long long)blocks_for(batch_mur_count(g.nx, g.ny, g.nz, g.boundary == 1), 256),
-        (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + s->lz - 1) / s->lz),
+        (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) *
+            ((g.nz + s->lz - 1) / s->lz),
         s->power_cap > 0 ? kBatchPowerBlocks : 0,
         (long long)((s->nkeys + 1 + kScanBlock - 1) / kScanBlock),
         s->np > 0 ? (long long)blocks_for(s->np, 256) : 0};
@@ -1977,7 +2050,7 @@ mithra_status capture_fused_typed(mithra_batch* b) {
   const int npg = (M + kPushGroup - 1) / kPushGroup;
   if (st == MITHRA_OK)
     st = grow(b, reinterpret_cast<void**>(&b->d_pref), &b->pref_bytes,
-              sizeof(int) * (size_t)(M + 2 * npg));
+              sizeof(int) * (size_t)(2 * M + 3 * npg));
   // block prefixes of the boundary and update phases, restarted at 0 for
   // each group of kZGroup members (M + 1 per group's entries)
   const int ngroups = (M + kZGroup - 1) / kZGroup;
@@ -2011,6 +2084,12 @@ mithra_status capture_fused_typed(mithra_batch* b) {
                         : k_push_tiled<true, T, U, false, true>)
                    : (lo ? k_push_tiled<false, T, U, kAnyLo, true>
                          : k_push_tiled<false, T, U, false, true>);
+  auto ksparse = opt ? (lo ? k_push_sparse<true, T, U, kAnyLo, true>
+                           : k_push_sparse<true, T, U, false, true>)
+                     : (lo ? k_push_sparse<false, T, U, kAnyLo, true>
+                           : k_push_sparse<false, T, U, false, true>);
+  bool sparse = false;
+  for (const BatchMember<T, U>& m : tab) sparse = sparse || m.sparse_below > 0;
   if (cudaFuncSetAttribute(kpush, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
       cudaSuccess)
     return bfail(b, MITHRA_ECUDA, "batched particle step: shared memory attribute");
@@ -2062,9 +2141,11 @@ mithra_status capture_fused_typed(mithra_batch* b) {
     // (their arguments in the launch's parameter space)
     for (int g0 = 0; g0 < M; g0 += kPushGroup) {
       const int Mg = std::min(kPushGroup, M - g0);
-      int* pref = b->d_pref + g0 + 2 * (g0 / kPushGroup);  // Mg + 1 entries, then the counter
-      int* work = pref + Mg + 1;
-      kb_tile_prefix<T, U><<<1, 1024, 0, q>>>(mem + g0, Mg, pref, work);
+      // Mg + 1 entries of each prefix, then the counter
+      int* pref = b->d_pref + 2 * g0 + 3 * (g0 / kPushGroup);
+      int* spref = pref + Mg + 1;
+      int* work = spref + Mg + 1;
+      kb_tile_prefix<T, U><<<1, 1024, 0, q>>>(mem + g0, Mg, pref, spref, work);
       PushParams<T, U, true> prm;
       for (int k = 0; k < Mg; ++k) {
         prm.m[k] = push_args_of(tab[(size_t)t * M + g0 + k]);
@@ -2072,8 +2153,10 @@ mithra_status capture_fused_typed(mithra_batch* b) {
         prm.box_d[k] = maps[(size_t)t * M + g0 + k].box_d;
       }
       prm.pref = pref;
+      prm.spref = spref;
       prm.work = work;
       prm.M = Mg;
+      if (sparse) ksparse<<<sparse_grid(b->sims[0]->n_sm), kSparseThreads, 0, q>>>(prm);
       kpush<<<b->push_grid, kPushThreads, smem, q>>>(prm);
     }
     kb_scan_partials<T, U><<<total(kBPScan), kScanBlock, 0, q>>>(mem, dblk + kBPScan * (M + 1), M);

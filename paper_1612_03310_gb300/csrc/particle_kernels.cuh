@@ -586,22 +586,25 @@ __global__ void k_deposit_rho(PicP<T> p, Parts<T, U> P, long long np, V4<T>* __r
   deposit_cic(p, src, i, j, k, P.fx[q], P.fy[q], P.fz[q], (T)0, (T)0, (T)0, p.qV);
 }
 
-// Block-wide exclusive scan of one int per thread (blockDim a multiple of 32,
-// at most 1024); *total receives the block sum.  Uses ws[32] shared ints.
-__device__ inline int block_exclusive_scan(int v, int* ws, int* total) {
+// Block-wide exclusive scan of one value per thread (blockDim a multiple of
+// 32, at most 1024); *total receives the block sum.  Uses ws[32] shared
+// values.  V: int, or a 64-bit word of two 32-bit sums (lo, hi; neither
+// overflows), which scans both at once.
+template <typename V>
+__device__ inline V block_exclusive_scan(V v, V* ws, V* total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  int incl = v;
+  V incl = v;
   for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    const V t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += t;
   }
   __syncthreads();
   if (lane == 31) ws[wid] = incl;
   __syncthreads();
   if (wid == 0) {
-    int w = (lane < (int)(blockDim.x >> 5)) ? ws[lane] : 0;
+    V w = (lane < (int)(blockDim.x >> 5)) ? ws[lane] : 0;
     for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, w, o);
+      const V t = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += t;
     }
     ws[lane] = w;  // inclusive over warps
@@ -611,94 +614,135 @@ __device__ inline int block_exclusive_scan(int v, int* ws, int* total) {
   return incl - v + (wid > 0 ? ws[wid - 1] : 0);
 }
 
-// Exclusive scan of the per-tile counts in two coalesced passes over blocks of
-// kScanBlock entries.  Pass 1 writes each block's sums (particles, dense
-// tiles, sparse tiles).  Pass 2 scans those sums, then its block: offset[t]
-// (offset[nkeys+1] = total), the list of non-empty tiles (key < nkeys; key
-// nkeys holds the lost particles) for the tiled particle kernel -- tiles with
-// at least sparse_below particles first (dense), then the others (sparse),
-// each group in key order -- the reset counts, and, in block 0, the two tile
-// counts, the reset work counters and (advance != 0: the last kernel of a
-// step) the step counter.  sparse_below = 0 lists every tile as dense.
-constexpr int kScanBlock = 1024;
+typedef unsigned long long Pair;  // two 32-bit sums of a scan
+__host__ __device__ inline Pair pair_of(int lo, int hi) {
+  return (Pair)(unsigned)lo | ((Pair)(unsigned)hi << 32);
+}
+__host__ __device__ inline int pair_lo(Pair p) { return (int)(unsigned)p; }
+__host__ __device__ inline int pair_hi(Pair p) { return (int)(unsigned)(p >> 32); }
 
-__device__ inline void tile_class(int c, int t, int nkeys, int sparse_below, int* dense,
-                                  int* sparse) {
+// Exclusive scan of the per-tile counts in two coalesced passes over blocks of
+// kScanBlock entries.  Pass 1 writes each block's sums (particles, units,
+// dense tiles, sparse tiles).  Pass 2 scans those sums, then its block:
+// offset[t] (offset[nkeys+1] = total), the list of non-empty tiles (key <
+// nkeys; key nkeys holds the lost particles) for the tiled particle kernel --
+// tiles with at least sparse_below particles first (dense), then the others
+// (sparse), each group in key order -- the dense tiles' work units, the reset
+// counts, and, in block 0, the two tile counts, the reset work counters and
+// (advance != 0: the last kernel of a step) the step counter.  sparse_below =
+// 0 lists every tile as dense.
+//
+// A unit is what one CTA of the particle step takes at a time: a tile, or a
+// run of at most `chunk` of its particles' slots, so that a few heavy tiles
+// (a short bunch: 3000 particles a tile in a hundred tiles) spread over the
+// device instead of keeping one CTA each busy.  units[0].x is their number,
+// units[1 + w] = {tile, first slot, end slot, 0}.
+//
+// kRestored: the counts come from a restored offset array instead (the lists
+// are rebuilt for this simulation's own chunk and threshold; offset, count
+// and the step counter stay as they are).
+constexpr int kScanBlock = 1024;
+constexpr int kMinChunk = 256;  // slots of the smallest unit of a split tile
+
+__device__ inline void tile_class(int c, int t, int nkeys, int sparse_below, int chunk,
+                                  int* dense, int* sparse, int* units) {
   const bool nonempty = c > 0 && t < nkeys;
   *dense = (nonempty && c >= sparse_below) ? 1 : 0;
   *sparse = (nonempty && c < sparse_below) ? 1 : 0;
+  *units = *dense ? (c + chunk - 1) / chunk : 0;
 }
 
-__device__ __forceinline__ void scan_partials_body(const int* __restrict__ count, int nkeys,
-                                                   int sparse_below, int4* __restrict__ part,
-                                                   int bidx) {
-  __shared__ int ws[32];
+template <bool kRestored>
+__device__ inline int tile_count(const int* __restrict__ count, const int* __restrict__ offset,
+                                 int t, int nkeys) {
+  if (t > nkeys) return 0;
+  return kRestored ? offset[t + 1] - offset[t] : count[t];
+}
+
+template <bool kRestored = false>
+__device__ __forceinline__ void scan_partials_body(const int* __restrict__ count,
+                                                   const int* __restrict__ offset, int nkeys,
+                                                   int sparse_below, int chunk,
+                                                   int4* __restrict__ part, int bidx) {
+  __shared__ Pair ws[32];
   const int t = bidx * kScanBlock + threadIdx.x;
-  const int c = (t <= nkeys) ? count[t] : 0;
-  int dn, sp;
-  tile_class(c, t, nkeys, sparse_below, &dn, &sp);
-  int tot, nd, ns;
-  block_exclusive_scan(c, ws, &tot);
-  block_exclusive_scan(dn, ws, &nd);
-  block_exclusive_scan(sp, ws, &ns);
-  if (threadIdx.x == 0) part[bidx] = make_int4(tot, nd, ns, 0);
+  const int c = tile_count<kRestored>(count, offset, t, nkeys);
+  int dn, sp, un;
+  tile_class(c, t, nkeys, sparse_below, chunk, &dn, &sp, &un);
+  Pair cu, ds;
+  block_exclusive_scan(pair_of(c, un), ws, &cu);
+  block_exclusive_scan(pair_of(dn, sp), ws, &ds);
+  if (threadIdx.x == 0)
+    part[bidx] = make_int4(pair_lo(cu), pair_hi(cu), pair_lo(ds), pair_hi(ds));
 }
 
+template <bool kRestored>
 __global__ void __launch_bounds__(kScanBlock) k_scan_partials(const int* __restrict__ count,
+                                                              const int* __restrict__ offset,
                                                               int nkeys, int sparse_below,
+                                                              int chunk,
                                                               int4* __restrict__ part) {
-  scan_partials_body(count, nkeys, sparse_below, part, blockIdx.x);
+  scan_partials_body<kRestored>(count, offset, nkeys, sparse_below, chunk, part, blockIdx.x);
 }
 
+template <bool kRestored = false>
 __device__ __forceinline__ void scan_final_body(int* __restrict__ count, int* __restrict__ offset,
-                                                int* __restrict__ tiles, int nkeys,
-                                                int sparse_below, const int4* __restrict__ part,
-                                                int nblocks, StepState* __restrict__ st,
-                                                int advance, int bidx) {
-  __shared__ int ws[32];
-  __shared__ int base[3], total[3];
+                                                int* __restrict__ tiles, int4* __restrict__ units,
+                                                int nkeys, int sparse_below, int chunk,
+                                                const int4* __restrict__ part, int nblocks,
+                                                StepState* __restrict__ st, int advance,
+                                                int bidx) {
+  __shared__ Pair ws[32];
+  __shared__ Pair base[2], total[2];
   // bases of this block from the block sums (nblocks <= kScanBlock)
   const int4 pv = (threadIdx.x < nblocks) ? part[threadIdx.x] : make_int4(0, 0, 0, 0);
-  int all_c, all_d, all_s;
-  const int bc = block_exclusive_scan(pv.x, ws, &all_c);
-  const int bd = block_exclusive_scan(pv.y, ws, &all_d);
-  const int bs = block_exclusive_scan(pv.z, ws, &all_s);
-  if (threadIdx.x == bidx) { base[0] = bc; base[1] = bd; base[2] = bs; }
-  if (threadIdx.x == 0) { total[0] = all_c; total[1] = all_d; total[2] = all_s; }
+  Pair all_cu, all_ds;
+  const Pair bcu = block_exclusive_scan(pair_of(pv.x, pv.y), ws, &all_cu);
+  const Pair bds = block_exclusive_scan(pair_of(pv.z, pv.w), ws, &all_ds);
+  if (threadIdx.x == bidx) { base[0] = bcu; base[1] = bds; }
+  if (threadIdx.x == 0) { total[0] = all_cu; total[1] = all_ds; }
   __syncthreads();
   const int t = bidx * kScanBlock + threadIdx.x;
-  const int c = (t <= nkeys) ? count[t] : 0;
-  int dn, sp;
-  tile_class(c, t, nkeys, sparse_below, &dn, &sp);
-  int dummy;
-  const int off = base[0] + block_exclusive_scan(c, ws, &dummy);
-  const int sd = base[1] + block_exclusive_scan(dn, ws, &dummy);
-  const int ss = total[1] + base[2] + block_exclusive_scan(sp, ws, &dummy);
+  const int c = tile_count<kRestored>(count, offset, t, nkeys);
+  int dn, sp, un;
+  tile_class(c, t, nkeys, sparse_below, chunk, &dn, &sp, &un);
+  Pair dummy;
+  const Pair cu = base[0] + block_exclusive_scan(pair_of(c, un), ws, &dummy);
+  const Pair ds = base[1] + block_exclusive_scan(pair_of(dn, sp), ws, &dummy);
   if (t <= nkeys) {
-    offset[t] = off;
-    count[t] = 0;
-    if (dn) tiles[sd] = t;
-    if (sp) tiles[ss] = t;
+    const int off = pair_lo(cu);
+    if (!kRestored) {
+      offset[t] = off;
+      count[t] = 0;
+    }
+    if (dn) tiles[pair_lo(ds)] = t;
+    if (sp) tiles[pair_lo(total[1]) + pair_hi(ds)] = t;
+    for (int w = 0; w < un; ++w)
+      units[1 + pair_hi(cu) + w] =
+          make_int4(t, off + w * chunk, off + min(c, (w + 1) * chunk), 0);
   }
   if (bidx == 0 && threadIdx.x == 0) {
-    offset[nkeys + 1] = total[0];
-    st->n_tiles = total[1];
-    st->n_sparse = total[2];
+    if (!kRestored) offset[nkeys + 1] = pair_lo(total[0]);
+    units[0] = make_int4(pair_hi(total[0]), 0, 0, 0);
+    st->n_tiles = pair_lo(total[1]);
+    st->n_sparse = pair_hi(total[1]);
     st->work = 0;
     st->work_sparse = 0;
     if (advance) st->n += 1;
   }
 }
 
+template <bool kRestored>
 __global__ void __launch_bounds__(kScanBlock) k_scan_final(int* __restrict__ count,
                                                            int* __restrict__ offset,
-                                                           int* __restrict__ tiles, int nkeys,
-                                                           int sparse_below,
+                                                           int* __restrict__ tiles,
+                                                           int4* __restrict__ units, int nkeys,
+                                                           int sparse_below, int chunk,
                                                            const int4* __restrict__ part,
                                                            int nblocks, StepState* __restrict__ st,
                                                            int advance) {
-  scan_final_body(count, offset, tiles, nkeys, sparse_below, part, nblocks, st, advance,
-                  blockIdx.x);
+  scan_final_body<kRestored>(count, offset, tiles, units, nkeys, sparse_below, chunk, part,
+                             nblocks, st, advance, blockIdx.x);
 }
 
 // The re-sort: slot offset[key] + rank of the next step's tile order gets

@@ -1,7 +1,8 @@
 // tile_push.cuh -- particle step by cell tiles.
 //
-// A persistent CTA takes dense 8^3-cell tiles from the list the last re-sort
-// produced.  For each tile it
+// A persistent CTA takes work units (a dense 8^3-cell tile, or a run of the
+// particles of a heavy one) from the list the last re-sort produced.  For
+// each it
 //   1. loads psi^{n+1} and the increment D over the vertices
 //      [t0 - 1, t0 + 9]^3 (11^3, two TMA box loads, one mbarrier);
 //   2. evaluates E and B at t = (n+1/2) dt at the tile's 9^3 vertices
@@ -135,7 +136,7 @@ __device__ inline void deposit_tile(const PicP<T>& p, T* __restrict__ sJ,
 // contribution is w q/V with a CIC weight w in [0, 1], so the block sums the
 // integers hi = rint(w 2^b) and lo = rint((w 2^b - hi) 2^b) with int32
 // shared atomics (native, unlike FP32 shared atomics), b = min(21, 30 -
-// ceil(log2 n_t)) for the tile's n_t particles: neither sum can overflow
+// ceil(log2 n_t)) for the unit's n_t particles: neither sum can overflow
 // (n_t 2^b <= 2^30), one contribution is resolved to 2^-2b q/V, and the sums
 // do not depend on the order of the atomics.  Rounding to an integer by
 // adding 1.5 2^23, exact for |x| < 2^22 (w 2^b <= 2^21; the products by
@@ -156,7 +157,7 @@ __device__ inline void deposit_rho_fixed(const PicP<T>& p, int* __restrict__ hi,
                                          int j0, int k0, int i, int j, int k, T fx, T fy, T fz,
                                          float sb) {
   const int li = i - (i0 - 1), lj = j - (j0 - 1), lk = k - (k0 - 1);
-  if (sb == 0.0f || li < 0 || li > kTP - 2 || lj < 0 || lj > kTP - 2 || lk < 0 ||
+  if (li < 0 || li > kTP - 2 || lj < 0 || lj > kTP - 2 || lk < 0 ||
       lk > kTP - 2) {
     deposit_cic(p, src, i, j, k, fx, fy, fz, (T)0, (T)0, (T)0, p.qV);
     return;
@@ -252,7 +253,7 @@ __device__ inline void tile_origin(const PicP<T>& p, int tile, int* i0, int* j0,
 // member by pref, one counter hands out.
 constexpr int kPushGroup = 30;  // 30 x (792 + 256) B (FP64) of the 32 KB parameter space
 
-// Member of tile number w of a batch group: pref[m] <= w < pref[m+1].
+// Member of unit number w of a batch group: pref[m] <= w < pref[m+1].
 __device__ inline int member_of_tile(const int* __restrict__ pref, int M, int w) {
   int lo = 0, hi = M - 1;
   while (lo < hi) {
@@ -277,10 +278,34 @@ struct PushParams<T, U, true> {
   CUtensorMap box[kPushGroup];    // the members' psi^{n+1}, 11^3 boxes
   CUtensorMap box_d[kPushGroup];  // their increments
   PushArgs<T, U> m[kPushGroup];
-  const int* pref;  // pref[0 .. M]: tiles before each member
-  int* work;        // tile counter
+  const int* pref;   // pref[0 .. M]: units before each member
+  const int* spref;  // spref[0 .. M]: sparse tiles before each member
+  int* work;         // unit counter
   int M;
 };
+
+// Source-tile flags (StencilP::dirty): the deposits mark the flags of the
+// next update -- a tile's 27 neighbours, which hold every vertex a particle
+// of the tile deposits to while its end and mid-point cells stay within
+// [t0 - 8, t0 + 14] on each axis (t0 the tile's first cell); a deposit beyond
+// that sets src_all of the next parity instead.
+template <typename T, typename U>
+__device__ inline void mark_tile(const PushArgs<T, U>& a, int tile, int r) {  // neighbour r of 27
+  const PicP<T>& p = a.p;
+  const int tx = tile % p.ntx + r % 3 - 1, ty = (tile / p.ntx) % p.nty + (r / 3) % 3 - 1,
+            tz = tile / (p.ntx * p.nty) + r / 9 - 1;
+  if (tx >= 0 && tx < p.ntx && ty >= 0 && ty < p.nty && tz >= 0 && tz < p.ntz)
+    a.dirty[(size_t)(1 - a.cur) * 4 * a.dirty_words + ((size_t)tz * p.nty + ty) * p.ntx + tx] = 1;
+}
+template <typename T, typename U>
+__device__ inline void far_deposit(const PushArgs<T, U>& a, int i0, int j0, int k0, int i, int j,
+                                   int k) {
+  if ((unsigned)(i - i0 + 8) > 22u || (unsigned)(j - j0 + 8) > 22u ||
+      (unsigned)(k - k0 + 8) > 22u)
+    a.st->src_all[1 - a.cur] = 1;
+}
+
+constexpr int kMaxFrames = 16;  // undulator frames kept per tile (sub-steps)
 
 template <bool kOpt, typename T, typename U, bool kLo = false, bool kBatch = false>
 __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
@@ -316,7 +341,6 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   int* sRh = reinterpret_cast<int*>(sP);
   int* sRl = sRh + kTPC;
   __shared__ int s_tile;
-  constexpr int kMaxFrames = 16;
   __shared__ UndFrame<T> s_frame[kMaxFrames];  // undulator frames of the tile
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -329,30 +353,13 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   // before any global access, for it to complete (a no-op otherwise)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   uint32_t phase = 0;
-  // Source-tile flags (StencilP::dirty): the array this step's potential
-  // update read is cleared, and the deposits mark the other -- a tile's 27
-  // neighbours, which hold every vertex a particle of the tile deposits to
-  // while its end and mid-point cells stay within [t0 - 8, t0 + 14] on each
-  // axis (t0 the tile's first cell); a deposit beyond that sets src_all of
-  // the next parity instead.
-  auto clear_flags = [&](const PushArgs<T, U>& a) {
+  // Source-tile flags: the array this step's potential update read is
+  // cleared, and the deposits mark the other (mark_tile, far_deposit)
+  // (done by CTA b of the nb that share the simulation)
+  auto clear_flags = [&](const PushArgs<T, U>& a, int b, int nb) {
     unsigned* f = reinterpret_cast<unsigned*>(a.dirty) + (size_t)a.cur * a.dirty_words;
-    for (int w = blockIdx.x * blockDim.x + tid; w < a.dirty_words; w += gridDim.x * blockDim.x)
-      f[w] = 0u;
-    if (blockIdx.x == 0 && tid == 0) a.st->src_all[a.cur] = 0;
-  };
-  auto mark_tile = [&](const PushArgs<T, U>& a, int tile, int r) {  // neighbour r of 27
-    const PicP<T>& p = a.p;
-    const int tx = tile % p.ntx + r % 3 - 1, ty = (tile / p.ntx) % p.nty + (r / 3) % 3 - 1,
-              tz = tile / (p.ntx * p.nty) + r / 9 - 1;
-    if (tx >= 0 && tx < p.ntx && ty >= 0 && ty < p.nty && tz >= 0 && tz < p.ntz)
-      a.dirty[(size_t)(1 - a.cur) * 4 * a.dirty_words + ((size_t)tz * p.nty + ty) * p.ntx + tx] =
-          1;
-  };
-  auto far_deposit = [&](const PushArgs<T, U>& a, int i0, int j0, int k0, int i, int j, int k) {
-    if ((unsigned)(i - i0 + 8) > 22u || (unsigned)(j - j0 + 8) > 22u ||
-        (unsigned)(k - k0 + 8) > 22u)
-      a.st->src_all[1 - a.cur] = 1;
+    for (int w = b * blockDim.x + tid; w < a.dirty_words; w += nb * blockDim.x) f[w] = 0u;
+    if (b == 0 && tid == 0) a.st->src_all[a.cur] = 0;
   };
   // the particle at position pos of the state buffer into this thread's
   // slot, and the position of the slot after it (qn, when below end) into
@@ -371,20 +378,20 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
     cp_async_commit();
   };
   // the slots after the last tile's (particles lost before this step): moved
-  // to the output buffer, their bucket kept
-  auto lost_tail = [&](const PushArgs<T, U>& a) {
+  // to the output buffer, their bucket kept, by CTA b of nb
+  auto lost_tail = [&](const PushArgs<T, U>& a, int b, int nb) {
     const int nk = a.p.nkeys;
-    for (long long q = a.offset[nk] + (long long)blockIdx.x * blockDim.x + tid; q < a.np;
-         q += (long long)gridDim.x * blockDim.x) {
+    for (long long q = a.offset[nk] + (long long)b * blockDim.x + tid; q < a.np;
+         q += (long long)nb * blockDim.x) {
       copy_particle(a.P, a.O, a.perm[q], q);
       a.key[q] = nk;
       a.rank[q] = bin_rank(a.count, nk);
     }
   };
-  // the dense tiles of one simulation's list, then its sparse tiles and lost
+  // the units of one simulation's list, then its sparse tiles and lost
   // tail (each written once; one simulation runs them straight through, a
   // batch member by member)
-  // one staged tile: entry t of the simulation's tile list
+  // one staged unit: entry t of the simulation's unit list
   auto dense = [&](const PushArgs<T, U>& a, const CUtensorMap* tmp, const CUtensorMap* tmd,
                    int t, double th) {
     const PicP<T>& p = a.p;
@@ -395,16 +402,13 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
     const Parts<T, U>& P = a.P;
     const Parts<T, U>& O = a.O;
     const int* const& perm = a.perm;
-    const int* const& offset = a.offset;
-    const int* const& tiles = a.tiles;
     int* const& count = a.count;
     int* const& key = a.key;
     int* const& rank = a.rank;
     long long* const& lost_ctr = a.lost_ctr;
     {
-      const int tile = tiles[t];
-      // the tile's particle range, loaded while the boxes are in flight
-      const int beg = offset[tile], end = offset[tile + 1];
+      const int4 unit = a.units[1 + t];
+      const int tile = unit.x, beg = unit.y, end = unit.z;
       int i0, j0, k0;
       tile_origin(p, tile, &i0, &j0, &k0);
       if (tid == 0) {
@@ -443,14 +447,13 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
       }
       __syncthreads();
       if (beg + tid < end) prefetch(P, perm, perm[beg + tid], beg + tid + kPushThreads, end);
-      // fixed-point scale 2^b of the FP32 charge block (0: tiles of more
-      // than 2^16 particles deposit rho in global memory)
+      // fixed-point scale 2^b of the FP32 charge block
       float sb = 0.0f;
       int bsh = 0;
       if (kF32) {
         const int nt = end - beg;
         bsh = min(21, 30 - (nt > 1 ? 32 - __clz(nt - 1) : 0));
-        if (nt <= 65536) sb = __int_as_float((127 + bsh) << 23);
+        sb = __int_as_float((127 + bsh) << 23);
         for (int c = tid; c < 2 * kTPC; c += blockDim.x) sRh[c] = 0;
       } else {
         for (int c = tid; c < 4 * kTPC; c += blockDim.x) sJ[c] = (T)0;
@@ -540,91 +543,35 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
       __syncthreads();
     }
   };
-  auto sparse = [&](const PushArgs<T, U>& a, int ntiles, double th) {
-    const PicP<T>& p = a.p;
-    StepState* const& st = a.st;
-    const V4<T>* const& pn = a.pn;
-    const V4<T>* const& D = a.D;
-    V4<T>* const& src = a.src;
-    const Parts<T, U>& P = a.P;
-    const Parts<T, U>& O = a.O;
-    const int* const& perm = a.perm;
-    const int* const& offset = a.offset;
-    const int* const& tiles = a.tiles;
-    int* const& count = a.count;
-    int* const& key = a.key;
-    int* const& rank = a.rank;
-    long long* const& lost_ctr = a.lost_ctr;
-    const long long& np = a.np;
-    // Sparse tiles: one warp per tile, no staging -- E and B evaluated at the
-    // vertices from global memory and the deposits added with global atomics.
-    // The whole CTA has left the loop above, so the E/B area is free for the
-    // warps' undulator frames.
-    const int nsparse = st->n_sparse;
-    if (nsparse > 0) {
-      const int lane = tid & 31;
-      UndFrame<T>* wf = reinterpret_cast<UndFrame<T>*>(sE) + (tid >> 5) * kMaxFrames;
-      for (;;) {
-        int w = 0;
-        if (lane == 0) w = atomicAdd(&st->work_sparse, 1);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= nsparse) break;
-        const int tile = tiles[ntiles + w];
-        int i0, j0, k0;
-        tile_origin(p, tile, &i0, &j0, &k0);
-        if (lane < 27) mark_tile(a, tile, lane);
-        __syncwarp();
-        for (int m = lane; m < p.n_sub && m < kMaxFrames; m += 32)
-          wf[m] = und_frame(p, k0, th + m * p.dtb);
-        __syncwarp();
-        const int beg = offset[tile], end = offset[tile + 1];
-        for (int q = beg + lane; q < end; q += 32) {
-          const long long pos = perm[q];
-          tile_particle<kOpt>(
-              p, O, q, count, key, rank, lost_ctr,
-              [&](int ci, int cj, int ck, const T* ff, T* E, T* B) {
-                gather_eb<kLo>(p, pn, D, ci, cj, ck, ff[0], ff[1], ff[2], E, B);
-              },
-              [&](int m, int kc, int* kref) {
-                *kref = k0;
-                return m < kMaxFrames ? wf[m] : und_frame(p, k0, th + m * p.dtb);
-              },
-              [&](bool rho, int i, int j, int k, const T* f, T jx, T jy, T jz, T q) {
-                far_deposit(a, i0, j0, k0, i, j, k);
-                deposit_cic(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz, q);
-              },
-              [&]() { return P.cell[pos]; },
-              [&](T* f, U* u) {
-                f[0] = P.fx[pos]; f[1] = P.fy[pos]; f[2] = P.fz[pos];
-                u[0] = P.ux[pos]; u[1] = P.uy[pos]; u[2] = P.uz[pos];
-              },
-              [&]() { return P.id[pos]; },
-              [&]() {});
-        }
-      }
-    }
-    // particles lost before this step sit at the tail of the sorted order (the
-    // bucket after the last tile); they keep that bucket in the re-sort
-    lost_tail(a);
-  };
   if constexpr (!kBatch) {
     const PushArgs<T, U>& a = prm.args;
-    clear_flags(a);
-    const int ntiles = a.st->n_tiles;
+    clear_flags(a, blockIdx.x, gridDim.x);
+    const int nunits = a.units[0].x;
     const double th = a.p.t0 + ((double)a.st->n + 0.5) * a.p.dt;
-    for (;;) {  // the CTA takes tiles from the list until none is left
+    for (;;) {  // the CTA takes units from the list until none is left
       if (tid == 0) s_tile = atomicAdd(&a.st->work, 1);
       __syncthreads();
       const int t = s_tile;
-      if (t >= ntiles) break;
+      if (t >= nunits) break;
       dense(a, &prm.tm_pn, &prm.tm_d, t, th);
     }
-    sparse(a, ntiles, th);
+    // particles lost before this step sit at the tail of the sorted order (the
+    // bucket after the last tile); they keep that bucket in the re-sort
+    lost_tail(a, blockIdx.x, gridDim.x);
   } else {
-    // the group's non-empty tiles (the dense and the sparse entries of each
-    // member's list, all staged) from one counter
+    // the group's units from one counter; the CTAs share the members for the
+    // flags and the lost tails
     const int M = prm.M;
-    for (int r = 0; r < M; ++r) clear_flags(prm.m[r]);
+    const int share = max((int)gridDim.x / M, 1);
+    auto each_member = [&](auto&& f) {
+      if ((int)gridDim.x >= M) {
+        const int b = blockIdx.x / M;
+        if (b < share) f(prm.m[blockIdx.x % M], b, share);
+      } else {
+        for (int r = blockIdx.x; r < M; r += gridDim.x) f(prm.m[r], 0, 1);
+      }
+    };
+    each_member(clear_flags);
     for (;;) {
       if (tid == 0) s_tile = atomicAdd(prm.work, 1);
       __syncthreads();
@@ -636,7 +583,84 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
       dense(a, &prm.box[mi], &prm.box_d[mi], w - prm.pref[mi], th);
     }
     // the particles each member lost before this step keep their bucket
-    for (int r = 0; r < M; ++r) lost_tail(prm.m[r]);
+    each_member(lost_tail);
+  }
+}
+
+// A sparse tile, one warp: no staging -- E and B evaluated at the vertices
+// from global memory, the deposits added with global atomics.  wf: the
+// warp's kMaxFrames undulator frames.
+template <bool kOpt, typename T, typename U, bool kLo>
+__device__ inline void push_sparse_tile(const PushArgs<T, U>& a, int tile, double th,
+                                              UndFrame<T>* wf) {
+  const PicP<T>& p = a.p;
+  const V4<T>* const& pn = a.pn;
+  const V4<T>* const& D = a.D;
+  V4<T>* const& src = a.src;
+  const Parts<T, U>& P = a.P;
+  const int lane = threadIdx.x & 31;
+  int i0, j0, k0;
+  tile_origin(p, tile, &i0, &j0, &k0);
+  if (lane < 27) mark_tile(a, tile, lane);
+  __syncwarp();
+  for (int m = lane; m < p.n_sub && m < kMaxFrames; m += 32)
+    wf[m] = und_frame(p, k0, th + m * p.dtb);
+  __syncwarp();
+  const int beg = a.offset[tile], end = a.offset[tile + 1];
+  for (int q = beg + lane; q < end; q += 32) {
+    const long long pos = a.perm[q];
+    tile_particle<kOpt>(
+        p, a.O, q, a.count, a.key, a.rank, a.lost_ctr,
+        [&](int ci, int cj, int ck, const T* ff, T* E, T* B) {
+          gather_eb<kLo>(p, pn, D, ci, cj, ck, ff[0], ff[1], ff[2], E, B);
+        },
+        [&](int m, int kc, int* kref) {
+          *kref = k0;
+          return m < kMaxFrames ? wf[m] : und_frame(p, k0, th + m * p.dtb);
+        },
+        [&](bool rho, int i, int j, int k, const T* f, T jx, T jy, T jz, T q) {
+          far_deposit(a, i0, j0, k0, i, j, k);
+          deposit_cic(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz, q);
+        },
+        [&]() { return P.cell[pos]; },
+        [&](T* f, U* u) {
+          f[0] = P.fx[pos]; f[1] = P.fy[pos]; f[2] = P.fz[pos];
+          u[0] = P.ux[pos]; u[1] = P.uy[pos]; u[2] = P.uz[pos];
+        },
+        [&]() { return P.id[pos]; },
+        [&]() {});
+  }
+}
+
+// The sparse tiles of one simulation or of a batch group, one warp each,
+// strided over the grid.  A kernel of its own beside k_push_tiled (other
+// tiles, the same counters and atomics): in that kernel its registers cost
+// the unit loop spills (44 against 24 bytes in the FP32 forms).
+constexpr int kSparseThreads = 128;
+
+template <bool kOpt, typename T, typename U, bool kLo = false, bool kBatch = false>
+__global__ void __launch_bounds__(kSparseThreads)
+    k_push_sparse(const __grid_constant__ PushParams<T, U, kBatch> prm) {
+  __shared__ UndFrame<T> s_frames[kSparseThreads / 32][kMaxFrames];
+  UndFrame<T>* wf = s_frames[threadIdx.x >> 5];
+  const int w0 = blockIdx.x * (kSparseThreads / 32) + (threadIdx.x >> 5);
+  const int nw = gridDim.x * (kSparseThreads / 32);
+  auto time_of = [&](const PushArgs<T, U>& a) {
+    return a.p.t0 + ((double)a.st->n + 0.5) * a.p.dt;
+  };
+  if constexpr (!kBatch) {
+    const PushArgs<T, U>& a = prm.args;
+    const int nsparse = a.st->n_sparse, ntiles = a.st->n_tiles;
+    for (int w = w0; w < nsparse; w += nw)
+      push_sparse_tile<kOpt, T, U, kLo>(a, a.tiles[ntiles + w], time_of(a), wf);
+  } else {
+    const int nsparse = prm.spref[prm.M];
+    for (int w = w0; w < nsparse; w += nw) {
+      const int mi = member_of_tile(prm.spref, prm.M, w);
+      const PushArgs<T, U>& a = prm.m[mi];
+      push_sparse_tile<kOpt, T, U, kLo>(a, a.tiles[a.st->n_tiles + w - prm.spref[mi]], time_of(a),
+                                        wf);
+    }
   }
 }
 
