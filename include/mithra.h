@@ -390,7 +390,8 @@ mithra_status mithra_read_spectrum(mithra_sim* sim, double* dW_domega, int64_t* 
  *     2: register z-marching, a thread walks its column for lz planes with
  *     three planes' sums in registers.
  *   lz: planes per CTA of the marching forms (0: about two waves of CTAs for
- *     variant 1, 16 for variant 2).
+ *     variant 1; for variant 2 up to 16, fewer where the grid, or the batch
+ *     the simulation is in, would leave multiprocessors without work).
  *   push_variant 0: one thread per particle, E and B evaluated at the eight
  *     vertices from global memory; 1: persistent CTAs over 8^3-cell particle
  *     tiles with the potentials, E/B and the deposit block in shared memory.
@@ -403,8 +404,8 @@ mithra_status mithra_read_spectrum(mithra_sim* sim, double* dW_domega, int64_t* 
  *     grids of at least 16 tiles per persistent CTA, and every tile staged on
  *     smaller ones; 1: every tile staged).  Takes effect from the tile list of
  *     the next re-sort.
- * Defaults: stencil_variant 2 with lz 16 (the fastest form of the potential
- * update on every grid timed), push_variant 1 when the driver provides TMA
+ * Defaults: stencil_variant 2 with lz 0 (the fastest form of the potential
+ * update on every grid timed; mithra_get_tuning shows the run taken), push_variant 1 when the driver provides TMA
  * tensor maps (else 0), push_ctas_per_sm 0, push_sparse_below 0. */
 typedef struct {
     int32_t stencil_variant;

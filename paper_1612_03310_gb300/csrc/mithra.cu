@@ -113,7 +113,8 @@ struct mithra_sim {
   std::string err;
   // potential-update variant: 0 direct, 1 z-marching TMA tiles (needs tm)
   int stencil_variant = 0;
-  int lz = 0;  // planes per CTA of the marching form
+  int lz = 0;  // planes per CTA of the marching forms
+  bool lz_auto = true;  // register form: by the size of the work (plane_run)
   int march_resident = 608;  // marching CTAs resident on the device at once
   bool have_tm = false;
   CUtensorMap tm[2];      // psi buffers, plane boxes of the marching update
@@ -138,8 +139,8 @@ struct mithra_sim {
 };
 
 void batch_mark_dirty(mithra_batch* b);  // defined with the batch
-// particles of all members of a batch
-void batch_totals(const mithra_batch* b, int64_t* particles);
+// particles and column planes (32 x 8 column tiles times planes) of a batch
+void batch_totals(const mithra_batch* b, int64_t* particles, int64_t* column_planes);
 
 namespace {
 
@@ -423,9 +424,29 @@ int64_t unit_entries(int64_t np, int64_t nkeys) { return 1 + nkeys + np / kMinCh
 // Particles that share the device with this simulation's: its batch's, or its
 // own.
 int64_t particles_beside(const mithra_sim* s) {
-  int64_t np = s->np;
-  if (s->in_batch) batch_totals(s->in_batch, &np);
+  int64_t np = s->np, planes = 0;
+  if (s->in_batch) batch_totals(s->in_batch, &np, &planes);
   return np;
+}
+
+int64_t column_planes(const mithra_grid& g) {
+  return (int64_t)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * g.nz;
+}
+
+// Planes per CTA of the register z-marching update: the caller's, or the
+// longest run up to 16 (a run reads two planes more than it updates) that
+// still gives every multiprocessor three CTAs; FP64 stops at 2, its
+// arithmetic and not its latency being the bound.  Measured potential scope:
+// 32 x 32 x 64 cells 21 us at 16 planes (16 CTAs), 12 us at 1; in FP64 132 and
+// 40 us (2 planes); 64 x 64 x 256 cells 28 us at 16, 23 us at 8.
+int plane_run(const mithra_sim* s) {
+  if (!s->lz_auto) return s->lz;
+  int64_t np = 0, planes = column_planes(s->g);
+  if (s->in_batch) batch_totals(s->in_batch, &np, &planes);
+  const int least = s->prec == MITHRA_P64 ? 2 : 1;
+  int lz = 16;
+  while (lz > least && planes < (int64_t)lz * 3 * s->n_sm) lz /= 2;
+  return lz;
 }
 
 // Tiles below this many particles take the sparse path (0: none): the
@@ -611,7 +632,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
     else
       k_mur_boundary<false, T><<<mg, dim3(32, 8), 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S);
     if (s->stencil_variant == 2) {
-      const int lz = s->lz;
+      const int lz = plane_run(s);
       dim3 blk(32, 8, 1);
       dim3 grd((s->g.nx + 31) / 32, (s->g.ny + 7) / 8, (s->g.nz + lz - 1) / lz);
       if (L0 && fused)
@@ -1179,7 +1200,7 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
       mithra_status r = setup_push_grid<T, U>(s);
       return r == MITHRA_OK ? setup_march<T>(s) : r;
     });
-    s->lz = 16;
+    s->lz = plane_run(s);
     if (st != MITHRA_OK) {
       std::string msg = s->err;
       return bail(st, msg);
@@ -1689,7 +1710,10 @@ mithra_status mithra_set_tuning(mithra_sim* s, const mithra_tuning* t) {
     return fail(s, MITHRA_EINVAL,
                 "the marching update keeps single-float levels: not with compensated levels");
   s->stencil_variant = t->stencil_variant;
-  s->lz = t->lz > 0 ? t->lz : (t->stencil_variant == 2 ? 16 : default_lz(&s->g, s->march_resident));
+  // (the run mithra_get_tuning showed, set again, stays the library's choice)
+  s->lz_auto = t->stencil_variant == 2 && (t->lz == 0 || (s->lz_auto && t->lz == s->lz));
+  s->lz = t->lz > 0 ? t->lz
+                    : (s->lz_auto ? plane_run(s) : default_lz(&s->g, s->march_resident));
   s->push_variant = t->push_variant;
   s->push_ctas_per_sm = t->push_ctas_per_sm;
   s->push_sparse_below = t->push_sparse_below;
@@ -1883,9 +1907,12 @@ void batch_mark_dirty(mithra_batch* b) {
   if (b) b->dirty = true;
 }
 
-void batch_totals(const mithra_batch* b, int64_t* particles) {
-  *particles = 0;
-  for (const mithra_sim* s : b->sims) *particles += s->np;
+void batch_totals(const mithra_batch* b, int64_t* particles, int64_t* column_planes) {
+  *particles = *column_planes = 0;
+  for (const mithra_sim* s : b->sims) {
+    *particles += s->np;
+    *column_planes += ::column_planes(s->g);
+  }
 }
 
 namespace {
@@ -1975,7 +2002,7 @@ BatchMember<T, U> member_entry(mithra_sim* s, int c, int pb) {
   m.g0 = s->u.gamma0;
   m.b0 = std::sqrt(1.0 - 1.0 / (s->u.gamma0 * s->u.gamma0));
   m.np = s->np;
-  m.lz = s->lz;
+  m.lz = plane_run(s);
   m.power_plane = s->power_plane;
   m.nkeys = s->nkeys;
   m.scan_nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
@@ -2034,7 +2061,7 @@ mithra_status capture_fused_typed(mithra_batch* b) {
     const long long nb[kBPCount] = {
         (long long)blocks_for(batch_mur_count(g.nx, g.ny, g.nz, g.boundary == 1), 256),
         (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) *
-            ((g.nz + s->lz - 1) / s->lz),
+            ((g.nz + plane_run(s) - 1) / plane_run(s)),
         s->power_cap > 0 ? kBatchPowerBlocks : 0,
         (long long)((s->nkeys + 1 + kScanBlock - 1) / kScanBlock),
         s->np > 0 ? (long long)blocks_for(s->np, 256) : 0};
