@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kScanBlock) kb_scan_final(
   const int g = blockIdx.x;
   const int mi = member_of(blk, M, g);
   const BatchMember<T, U>& m = mem[mi];
-  scan_final_body(m.count, m.offset, m.tiles, m.units, m.nkeys, m.sparse_below, m.chunk,
+  scan_final_body(m.count, m.count_next, m.offset, m.tiles, m.units, m.nkeys, m.sparse_below, m.chunk,
                   m.scan_part, m.scan_nb, m.st, 1, g - blk[mi]);
 }
 

@@ -52,6 +52,7 @@ struct BatchMember {
   int* tiles;
   int4* units;
   int* count;
+  int* count_next;  // cleared for the next step (k_scan_final)
   int* key;
   int* rank;
   int4* scan_part;

@@ -51,6 +51,7 @@ struct mithra_sim {
   // (never true between API calls)
   cudaEvent_t ev_rs_fork = nullptr, ev_rs_join = nullptr;
   bool resort_pending = false;
+  int resort_parity = 0;  // level parity of that step
   int cur = 0;  // P[cur] holds the newest level
   int pb = 0;   // particle buffer in use
   void* P[2] = {nullptr, nullptr};  // psi ping-pong; P[cur] is the newest level
@@ -65,7 +66,10 @@ struct mithra_sim {
   int* perm = nullptr;
   int* key = nullptr;
   int* rank = nullptr;
-  int* count = nullptr;
+  // tile counts of the steps of either level parity: count[cur] is zero
+  // between steps, and the re-sort of a step clears the other.  One array
+  // cleared in place on grids of more keys than k_resort_small takes.
+  int* count[2] = {nullptr, nullptr};
   int* offset = nullptr;
   int* tiles = nullptr;  // non-empty tile list written by the scan
   int4* units = nullptr;  // the particle step's work units, written by the scan
@@ -469,14 +473,16 @@ unsigned sparse_grid(int n_sm) { return 8u * n_sm; }
 // Two-pass scan of the per-tile counts (see k_scan_final), on stream q
 // (default: the simulation's).
 template <bool kRestored = false>
-void launch_scan(mithra_sim* s, int advance, cudaStream_t q = nullptr) {
+void launch_scan(mithra_sim* s, int advance, int parity, cudaStream_t q = nullptr) {
   if (!q) q = s->stream;
+  int* const cnt = s->count[parity];
+  int* const next = s->count[1 - parity];
   const int nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
   const int below = sparse_below(s);
   const int chunk = unit_chunk(particles_beside(s), s->push_grid);
-  k_scan_partials<kRestored><<<nb, kScanBlock, 0, q>>>(s->count, s->offset, s->nkeys,
+  k_scan_partials<kRestored><<<nb, kScanBlock, 0, q>>>(cnt, s->offset, s->nkeys,
                                                        below, chunk, s->scan_part);
-  k_scan_final<kRestored><<<nb, kScanBlock, 0, q>>>(s->count, s->offset, s->tiles, s->units,
+  k_scan_final<kRestored><<<nb, kScanBlock, 0, q>>>(cnt, next, s->offset, s->tiles, s->units,
                                                     s->nkeys, below, chunk, s->scan_part,
                                                     nb, s->dstate, advance);
 }
@@ -569,12 +575,26 @@ void set_source_flags(const mithra_sim* s, int c, StencilP<T>* sp) {
   sp->nty = s->nty;
 }
 
-// The re-sort of the particle step just launched: scan of the tile counts
-// (it advances the device step counter) and the slot map, on stream q.
-void launch_resort(mithra_sim* s, cudaStream_t q) {
+bool small_resort(const mithra_sim* s) { return s->count[0] != s->count[1]; }
+
+// The re-sort of the particle step of level parity `parity` (it advances the
+// device step counter), on stream q: scan and slot map, in one kernel on
+// grids of few tiles.
+void launch_resort(mithra_sim* s, int parity, cudaStream_t q) {
+  if (small_resort(s)) {
+    // the scan's scope holds the whole re-sort, the slot map's is empty
+    { ProfScope none(s, K_SLOT_MAP); }
+    ProfScope ps(s, K_SCAN);
+    const unsigned nb = std::min<unsigned>(blocks_for(s->np, 4 * kSmallThreads), 2 * s->n_sm);
+    k_resort_small<<<nb, kSmallThreads, 0, q>>>(
+        s->count[parity], s->count[1 - parity], s->offset, s->tiles, s->units, s->nkeys,
+        sparse_below(s), unit_chunk(particles_beside(s), s->push_grid), s->dstate, s->np, s->key,
+        s->rank, s->perm);
+    return;
+  }
   {
     ProfScope ps(s, K_SCAN);
-    launch_scan(s, 1, q);
+    launch_scan(s, 1, parity, q);
   }
   ProfScope ps(s, K_SLOT_MAP);
   k_slot_map<<<blocks_for(s->np, 256 * kSlotPer), 256, 0, q>>>(s->np, s->key, s->rank,
@@ -592,7 +612,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
   if (overlap) {
     cudaEventRecord(s->ev_rs_fork, s->stream);
     cudaStreamWaitEvent(s->side, s->ev_rs_fork, 0);
-    launch_resort(s, s->side);
+    launch_resort(s, s->resort_parity, s->side);
     cudaEventRecord(s->ev_rs_join, s->side);
     s->resort_pending = false;
   }
@@ -738,7 +758,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         pa.offset = s->offset;
         pa.tiles = s->tiles;
         pa.units = s->units;
-        pa.count = s->count;
+        pa.count = s->count[s->cur];
         pa.key = s->key;
         pa.rank = s->rank;
         pa.lost_ctr = &s->dstate->n_lost;
@@ -770,7 +790,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
           if (lo) kern = opt ? k_push<true, T, U, true> : k_push<false, T, U, true>;
         if (!kern) return fail(s, MITHRA_EINVAL, "no particle-step form for this precision");
         kern<<<blocks_for(s->np, 256), 256, 0, s->stream>>>(pp, s->dstate, P1, Dn, S, A, B,
-                                                             s->perm, s->np, s->count, s->key,
+                                                             s->perm, s->np, s->count[s->cur], s->key,
                                                              s->rank, &s->dstate->n_lost);
         mark_sources_everywhere(s);  // this form marks no tiles
       }
@@ -787,17 +807,19 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
       cudaEventRecord(s->ev_join, s->side);
       cudaStreamWaitEvent(s->stream, s->ev_join, 0);
     }
-    if (defer && !s->profiling)
+    if (defer && !s->profiling) {
       s->resort_pending = true;
-    else
-      launch_resort(s, s->stream);
+      s->resort_parity = s->cur;
+    } else {
+      launch_resort(s, s->cur, s->stream);
+    }
     s->pb = 1 - s->pb;
   } else {
     if (branch) {
       cudaEventRecord(s->ev_join, s->side);
       cudaStreamWaitEvent(s->stream, s->ev_join, 0);
     }
-    launch_scan(s, 1);
+    launch_scan(s, 1, s->cur);
   }
   s->cur = 1 - s->cur;
   cudaError_t e = cudaGetLastError();
@@ -818,9 +840,9 @@ mithra_status init_particles(mithra_sim* s, const mithra_bunch* b) {
   Parts<T, U> A = parts_of<T, U>(s, 0), B = parts_of<T, U>(s, 1);
   long long* lost = &s->dstate->n_lost;
   k_init_particles<T, U><<<blocks_for(n, 256), 256, 0, s->stream>>>(
-      pp, n, d, d + n, d + 2 * n, d + 3 * n, d + 4 * n, d + 5 * n, A, s->count, s->key, s->rank,
-      lost);
-  launch_scan(s, 0);
+      pp, n, d, d + n, d + 2 * n, d + 3 * n, d + 4 * n, d + 5 * n, A, s->count[1 - s->cur], s->key,
+      s->rank, lost);
+  launch_scan(s, 0, 1 - s->cur);
   k_sort_particles<T, U><<<blocks_for(n, 256), 256, 0, s->stream>>>(A, B, n, s->key, s->rank,
                                                                     s->offset, s->perm);
   s->pb = 1;
@@ -1009,8 +1031,8 @@ void lab_of(const mithra_sim* s, int32_t kp, double t, double* t_lab, double* z_
 
 void free_all(mithra_sim* s) {
   if (s->stream) cudaStreamSynchronize(s->stream);
-  void* ptrs[] = {s->P[0], s->P[1], s->PL[0], s->PL[1], s->D, s->S, s->pbuf[0], s->pbuf[1], s->perm, s->key, s->rank, s->count,
-                  s->offset, s->tiles, s->units, s->dirty, s->scan_part, s->dstate, s->d_scalar, s->d_power_rec,
+  void* ptrs[] = {s->P[0], s->P[1], s->PL[0], s->PL[1], s->D, s->S, s->pbuf[0], s->pbuf[1], s->perm, s->key, s->rank, s->count[0],
+                  s->count[1] != s->count[0] ? s->count[1] : nullptr, s->offset, s->tiles, s->units, s->dirty, s->scan_part, s->dstate, s->d_scalar, s->d_power_rec,
                   s->d_spec_omega, s->d_spec_acc, s->d_spec_out, s->d_spec_samples,
                   s->d_bunch_rec, s->d_bunch_part};
   for (void* p : ptrs)
@@ -1063,6 +1085,7 @@ mithra_status mithra_footprint(const mithra_grid* grid, int64_t n_particles,
   b += 2 * (int64_t)particle_buffer_bytes(n_particles, precision);
   b += 3 * n_particles * (int64_t)sizeof(int);                   // slot map, key, rank
   b += 3 * (nkeys + 2) * (int64_t)sizeof(int);                   // count, offset, tiles
+  if (nkeys < kSmallKeys) b += (nkeys + 2) * (int64_t)sizeof(int);  // the other count array
   b += unit_entries(n_particles, nkeys) * (int64_t)sizeof(int4);  // particle-step units
   b += 8 * ((nkeys + 3) / 4);                                     // source-tile flags
   b += (nkeys / kScanBlock + 2) * (int64_t)sizeof(int4);         // scan block sums
@@ -1149,7 +1172,7 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
             dalloc((void**)&s->perm, sizeof(int) * (size_t)(np + 1)) &&
             dalloc((void**)&s->key, sizeof(int) * (size_t)(np + 1)) &&
             dalloc((void**)&s->rank, sizeof(int) * (size_t)(np + 1)) &&
-            dalloc((void**)&s->count, sizeof(int) * (size_t)(s->nkeys + 2)) &&
+            dalloc((void**)&s->count[0], sizeof(int) * (size_t)(s->nkeys + 2)) &&
             dalloc((void**)&s->offset, sizeof(int) * (size_t)(s->nkeys + 2)) &&
             dalloc((void**)&s->tiles, sizeof(int) * (size_t)(s->nkeys + 1)) &&
             dalloc((void**)&s->units, sizeof(int4) * (size_t)unit_entries(np, s->nkeys)) &&
@@ -1157,6 +1180,10 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
             dalloc((void**)&s->scan_part, sizeof(int4) * (size_t)(s->nkeys / kScanBlock + 2)) &&
             dalloc((void**)&s->dstate, sizeof(StepState)) &&
             dalloc((void**)&s->d_scalar, sizeof(double));
+  if (ok && s->nkeys < kSmallKeys)
+    ok = dalloc((void**)&s->count[1], sizeof(int) * (size_t)(s->nkeys + 2));
+  else
+    s->count[1] = s->count[0];
   const size_t lo_bytes = (size_t)ncell_of(grid) * sizeof(LoV4);
   if (ok && has_lo(precision))
     ok = dalloc(&s->PL[0], lo_bytes) && dalloc(&s->PL[1], lo_bytes);
@@ -1171,7 +1198,7 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
     if (l) cudaMemsetAsync(l, 0, lo_bytes, s->stream);
   cudaMemsetAsync(s->D, 0, field_bytes, s->stream);
   cudaMemsetAsync(s->S, 0, field_bytes, s->stream);
-  cudaMemsetAsync(s->count, 0, sizeof(int) * (size_t)(s->nkeys + 2), s->stream);
+  for (int* c : s->count) cudaMemsetAsync(c, 0, sizeof(int) * (size_t)(s->nkeys + 2), s->stream);
   cudaMemsetAsync(s->dstate, 0, sizeof(StepState), s->stream);
   cudaMemsetAsync(s->dirty, 0, 8 * (size_t)s->dirty_words, s->stream);
   mark_sources_everywhere(s);
@@ -1767,7 +1794,7 @@ std::vector<SnapPart> snap_parts(const mithra_sim* s) {
   }
   v.push_back({s->pbuf[s->pb], particle_buffer_bytes(s->np, s->prec)});
   v.push_back({s->perm, sizeof(int) * (size_t)s->np});
-  v.push_back({s->count, sizeof(int) * (size_t)(s->nkeys + 2)});
+  v.push_back({s->count[s->cur], sizeof(int) * (size_t)(s->nkeys + 2)});
   v.push_back({s->offset, sizeof(int) * (size_t)(s->nkeys + 2)});
   v.push_back({s->tiles, sizeof(int) * (size_t)(s->nkeys + 1)});
   v.push_back({s->dstate, sizeof(StepState)});
@@ -1825,7 +1852,7 @@ mithra_status mithra_restore(mithra_sim* s, const void* in) {
     p += part.bytes;
   }
   // the tile and unit lists for this simulation's own launch choices
-  if (s->np > 0) launch_scan<true>(s, 0);
+  if (s->np > 0) launch_scan<true>(s, 0, s->cur);
   mark_sources_everywhere(s);
   MCHECK(s, refresh_mirror(s));
   mithra_status st = sync_status(s);
@@ -1992,7 +2019,8 @@ BatchMember<T, U> member_entry(mithra_sim* s, int c, int pb) {
   m.offset = s->offset;
   m.tiles = s->tiles;
   m.units = s->units;
-  m.count = s->count;
+  m.count = s->count[c];
+  m.count_next = s->count[1 - c];
   m.key = s->key;
   m.rank = s->rank;
   m.scan_part = s->scan_part;

@@ -686,7 +686,8 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_partials(const int* __restr
 }
 
 template <bool kRestored = false>
-__device__ __forceinline__ void scan_final_body(int* __restrict__ count, int* __restrict__ offset,
+__device__ __forceinline__ void scan_final_body(const int* count, int* next,
+                                                int* __restrict__ offset,
                                                 int* __restrict__ tiles, int4* __restrict__ units,
                                                 int nkeys, int sparse_below, int chunk,
                                                 const int4* __restrict__ part, int nblocks,
@@ -713,7 +714,7 @@ __device__ __forceinline__ void scan_final_body(int* __restrict__ count, int* __
     const int off = pair_lo(cu);
     if (!kRestored) {
       offset[t] = off;
-      count[t] = 0;
+      next[t] = 0;
     }
     if (dn) tiles[pair_lo(ds)] = t;
     if (sp) tiles[pair_lo(total[1]) + pair_hi(ds)] = t;
@@ -733,7 +734,7 @@ __device__ __forceinline__ void scan_final_body(int* __restrict__ count, int* __
 }
 
 template <bool kRestored>
-__global__ void __launch_bounds__(kScanBlock) k_scan_final(int* __restrict__ count,
+__global__ void __launch_bounds__(kScanBlock) k_scan_final(const int* count, int* next,
                                                            int* __restrict__ offset,
                                                            int* __restrict__ tiles,
                                                            int4* __restrict__ units, int nkeys,
@@ -741,7 +742,7 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_final(int* __restrict__ cou
                                                            const int4* __restrict__ part,
                                                            int nblocks, StepState* __restrict__ st,
                                                            int advance) {
-  scan_final_body<kRestored>(count, offset, tiles, units, nkeys, sparse_below, chunk, part,
+  scan_final_body<kRestored>(count, next, offset, tiles, units, nkeys, sparse_below, chunk, part,
                              nblocks, st, advance, blockIdx.x);
 }
 
@@ -795,6 +796,83 @@ __global__ void __launch_bounds__(256) k_slot_map(long long np, const int* __res
     const long long q = q0 + (long long)u * blockDim.x;
     if (q < np) perm[(long long)offset[kk[u]] + rr[u]] = (int)q;
   }
+}
+
+// The whole re-sort (scan, lists and slot map) of a grid of at most
+// kSmallKeys keys in one launch: every block scans all the counts (16 KB from
+// L2 at most) into offsets in shared memory, then maps its share of the
+// particles; block 0 also writes the offsets, the lists and the step state.
+// The counts of the next step are the other of two arrays, so that clearing
+// it disturbs no block's scan.  What bounds the re-sort of a small grid is
+// launches and latency: by event pairs (some 5 us of each) three kernels took
+// 12 + 6 us and this one 8 on 32 x 32 x 64 cells with 4096 particles (129
+// keys), 13 + 7 and 12 on 64 x 64 x 256 with 262144 (2049 keys); at 6761
+// keys, where each thread walks 14, 13 + 8 and 19, so the line is drawn below.
+constexpr int kSmallPer = 8;  // keys a thread
+constexpr int kSmallThreads = 512;
+constexpr int kSmallKeys = kSmallPer * kSmallThreads;
+
+__global__ void __launch_bounds__(kSmallThreads, 2) k_resort_small(
+    const int* __restrict__ count, int* __restrict__ next, int* __restrict__ offset,
+    int* __restrict__ tiles, int4* __restrict__ units, int nkeys, int sparse_below, int chunk,
+    StepState* __restrict__ st, long long np, const int* __restrict__ key,
+    const int* __restrict__ rank, int* __restrict__ perm) {
+  __shared__ int s_off[kSmallKeys];
+  __shared__ Pair ws[32];
+  // (nkeys + 1) / 512 rounded up, 1 .. kSmallPer consecutive keys a thread
+  const int per = (nkeys + kSmallThreads) / kSmallThreads;
+  const int t0 = threadIdx.x * per;
+  // the thread's counts, kept in its own part of s_off until they become
+  // offsets
+  Pair cu = 0, ds = 0;
+#pragma unroll 8
+  for (int m = 0; m < per; ++m) {
+    const int t = t0 + m;
+    const int c = t <= nkeys ? count[t] : 0;
+    int dn, sp, un;
+    tile_class(c, t, nkeys, sparse_below, chunk, &dn, &sp, &un);
+    cu += pair_of(c, un);
+    ds += pair_of(dn, sp);
+    if (t <= nkeys) s_off[t] = c;
+  }
+  Pair total_cu, total_ds;
+  cu = block_exclusive_scan(cu, ws, &total_cu);
+  ds = block_exclusive_scan(ds, ws, &total_ds);
+  const bool lists = blockIdx.x == 0;
+  for (int m = 0; m < per; ++m) {
+    const int t = t0 + m;
+    if (t > nkeys) break;
+    const int c = s_off[t];
+    int dn, sp, un;
+    tile_class(c, t, nkeys, sparse_below, chunk, &dn, &sp, &un);
+    const int off = pair_lo(cu);
+    s_off[t] = off;
+    if (lists) {
+      offset[t] = off;
+      if (dn) tiles[pair_lo(ds)] = t;
+      if (sp) tiles[pair_lo(total_ds) + pair_hi(ds)] = t;
+      for (int w = 0; w < un; ++w)
+        units[1 + pair_hi(cu) + w] =
+            make_int4(t, off + w * chunk, off + min(c, (w + 1) * chunk), 0);
+    }
+    cu += pair_of(c, un);
+    ds += pair_of(dn, sp);
+  }
+  if (lists && threadIdx.x == 0) {
+    offset[nkeys + 1] = pair_lo(total_cu);
+    units[0] = make_int4(pair_hi(total_cu), 0, 0, 0);
+    st->n_tiles = pair_lo(total_ds);
+    st->n_sparse = pair_hi(total_ds);
+    st->work = 0;
+    st->work_sparse = 0;
+    st->n += 1;
+  }
+  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t <= nkeys; t += gridDim.x * blockDim.x)
+    next[t] = 0;
+  __syncthreads();
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < np;
+       q += (long long)gridDim.x * blockDim.x)
+    perm[(long long)s_off[key[q]] + rank[q]] = (int)q;
 }
 
 // Copy-out in the original particle order: FP64 positions from (cell, f).

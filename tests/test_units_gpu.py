@@ -1,0 +1,68 @@
+"""The particle step's work units and the one-kernel re-sort, at the sizes
+where they can go wrong: tiles of exactly one, a whole number and one more
+than a whole number of units, key counts around the scans' block sizes, the
+sparse tiles' kernel beside the units, an empty bunch; against the oracle."""
+import numpy as np
+import pytest
+
+from paper_1612_03310_gb300 import inputs
+from test_parity_gpu import C1_UND, M, compare_fields, compare_particles  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+# tolerances of the parity tests' single steps, for their reasons: sums of a
+# few FP32 roundings a step
+TOL = {"P64": (1e-10, 1e-10, 1e-9), "P32": (1e-5, 2e-5, 1e-5), "P32_U64": (1e-5, 2e-5, 1e-5)}
+
+
+def heavy_bunch(seed, g, counts):
+    """counts[m] particles in the m-th 8^3-cell tile (clear of the outer
+    cells), the rest of the grid empty."""
+    rng = np.random.default_rng(seed)
+    r = []
+    tiles = [(i, j, k) for k in range(g["nz"] // 8) for j in range(g["ny"] // 8)
+             for i in range(g["nx"] // 8)]
+    for (i, j, k), n in zip(tiles, counts):
+        lo = np.array([max(8 * c, 3) for c in (i, j, k)], float)
+        hi = np.array([min(8 * c + 8, v - 5) for c, v in zip((i, j, k), (g["nx"], g["ny"], g["nz"]))],
+                      float)
+        r.append(lo + (hi - lo) * rng.random((n, 3)))
+    r = np.concatenate(r)
+    u = 0.2 * rng.standard_normal((3, len(r)))
+    return dict(x=g["x0"] + r[:, 0] * g["dx"], y=g["y0"] + r[:, 1] * g["dy"],
+                z=g["z0"] + r[:, 2] * g["dz"], ux=u[0], uy=u[1], uz=u[2], q_macro=-1e-15)
+
+
+def check(M, orc, g, und, P, prec, steps, **tuning):  # noqa: F811
+    o = orc.OracleSim(g, und, P)
+    tf, tc, eps = TOL[prec]
+    with M.Simulation(dict(g, boundary=1), und, P, precision=getattr(M, prec)) as sim:
+        if tuning:
+            sim.set_tuning(**tuning)
+        for n in steps:
+            o.step(n)
+            sim.step(n)
+            sim.sync()
+            compare_fields(sim, o, tf, names=["Ex", "Ey", "Bz", "phi", "Jx", "Jz", "rho"])
+            compare_particles(sim, o, tc, eps)
+
+
+@pytest.mark.parametrize("prec", ["P64", "P32", "P32_U64"])
+@pytest.mark.parametrize("below", [0, 300])
+def test_split_tiles(M, orc, prec, below):  # noqa: F811
+    # units of 256 slots: one short of, exactly, and one over one and two
+    # units, a heavy tile, empty ones between; with below = 300 the light
+    # tiles go to the sparse tiles' kernel
+    g = inputs.random_grid(41, 32, 24, 24)
+    P = heavy_bunch(42, g, [255, 256, 257, 0, 511, 512, 513, 1, 0, 3000])
+    check(M, orc, g, dict(C1_UND, z_ent_lab=0.0), P, prec, (1, 4), push_sparse_below=below)
+
+
+@pytest.mark.parametrize("shape", [(8, 8, 8), (64, 64, 64), (24, 152, 72), (72, 56, 2056),
+                                   (128, 128, 128), (136, 128, 128)])
+def test_resort_key_counts(M, orc, shape):  # noqa: F811
+    # 1, 512 and 513 tiles (one and two keys a thread of the one-kernel
+    # re-sort), 16191 (two passes), 4096 (the two-pass limit) and 4352
+    g = inputs.random_grid(51, *shape)
+    P = inputs.random_particles(52, g, 3000, u_scale=0.2)
+    check(M, orc, g, dict(C1_UND, z_ent_lab=0.0), P, "P32_U64", (1, 4))
