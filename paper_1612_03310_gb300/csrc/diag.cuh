@@ -113,6 +113,15 @@ __global__ void k_bunch_final(const double* __restrict__ part, int nblocks,
 // F = (E'_x, E'_y, B'_x, B'_y) the lab transformation of k_power.
 constexpr int kMaxSpectrum = 64;
 
+// Four threads a vertex, one lab component f each, so that a warp's sums of a
+// wavelength are 512 contiguous bytes, four wavelengths' in flight at once; E
+// and B are evaluated by each of the four (the same addresses in a warp).
+// Bound by latency and, beyond some 30 wavelengths, by the 128 B a vertex and
+// wavelength through L2: 128 x 128 vertices, 16 wavelengths, 36 us with a
+// thread a vertex (63 blocks walking the sums 64 B apart), 20 us so (event
+// pairs, launch included).
+constexpr int kSpecFly = 4;
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_spectrum_accumulate(
     PicP<T> p, const V4<T>* __restrict__ pn, const V4<T>* __restrict__ D, int kp, double g0,
@@ -133,23 +142,34 @@ __global__ void __launch_bounds__(256) k_spectrum_accumulate(
   if (blockIdx.x == 0 && threadIdx.x == 0) *samples += 1;
   const int nvx = p.nx - 2;
   const long long nv = (long long)nvx * (p.ny - 2);
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < nv;
-       v += (long long)gridDim.x * blockDim.x) {
-    const int i = 1 + (int)(v % nvx), j = 1 + (int)(v / nvx);
-    T E[3], B[3];
-    eb_vertex(p, pn, D, cidx(i, j, kp, p.nx, p.nxy), E, B);
-    const double Ex = E[0], Ey = E[1], Bx = B[0], By = B[1];
-    const double F[4] = {g0 * (Ex + b0 * kC * By), g0 * (Ey - b0 * kC * Bx),
-                         g0 * (Bx - b0c * Ey), g0 * (By + b0c * Ex)};
-    for (int m = 0; m < nf; ++m) {
-      double* a = acc + ((long long)m * nv + v) * 8;
-      const double2 e = ph[m];
+  const long long w = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long v = w >> 2;
+  const int f = (int)(w & 3);
+  if (v >= nv) return;
+  const int i = 1 + (int)(v % nvx), j = 1 + (int)(v / nvx);
+  T E[3], B[3];
+  eb_vertex(p, pn, D, cidx(i, j, kp, p.nx, p.nxy), E, B);
+  const double Ex = E[0], Ey = E[1], Bx = B[0], By = B[1];
+  double F;
+  if (f == 0) F = g0 * (Ex + b0 * kC * By);
+  else if (f == 1) F = g0 * (Ey - b0 * kC * Bx);
+  else if (f == 2) F = g0 * (Bx - b0c * Ey);
+  else F = g0 * (By + b0c * Ex);
+  double2* a = reinterpret_cast<double2*>(acc) + w;
+  const long long stride = 4 * nv;
+  for (int m0 = 0; m0 < nf; m0 += kSpecFly) {
+    double2 s[kSpecFly];
 #pragma unroll
-      for (int f = 0; f < 4; ++f) {
-        a[2 * f] += F[f] * e.x;
-        a[2 * f + 1] += F[f] * e.y;
+    for (int m = 0; m < kSpecFly; ++m)
+      if (m0 + m < nf) s[m] = a[(m0 + m) * stride];
+#pragma unroll
+    for (int m = 0; m < kSpecFly; ++m)
+      if (m0 + m < nf) {
+        const double2 e = ph[m0 + m];
+        s[m].x += F * e.x;
+        s[m].y += F * e.y;
+        a[(m0 + m) * stride] = s[m];
       }
-    }
   }
 }
 

@@ -708,7 +708,9 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
   }
   if (s->power_cap > 0) {
     ProfScope ps(s, K_POWER);
-    k_power<T><<<64, 256, 0, dq>>>(pp, P1, Dn, s->power_plane, s->u.gamma0,
+    // without particles the two diagnostics run beside each other
+    cudaStream_t pq = s->np > 0 ? dq : s->stream;
+    k_power<T><<<64, 256, 0, pq>>>(pp, P1, Dn, s->power_plane, s->u.gamma0,
                                           std::sqrt(1.0 - 1.0 / (s->u.gamma0 * s->u.gamma0)),
                                           s->d_power_rec - s->power_first, s->dstate,
                                           s->power_first + s->power_cap, 1, &s->dstate->err);
@@ -717,7 +719,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
     ProfScope ps(s, K_SPECTRUM);
     const double g0 = s->u.gamma0;
     const long long nv = (long long)(s->g.nx - 2) * (s->g.ny - 2);
-    k_spectrum_accumulate<T><<<blocks_for(nv, 256), 256, 0, dq>>>(
+    k_spectrum_accumulate<T><<<blocks_for(4 * nv, 256), 256, 0, dq>>>(
         pp, P1, Dn, s->spec_plane, g0, std::sqrt(1.0 - 1.0 / (g0 * g0)),
         s->g.z0 + s->spec_plane * s->g.dz, s->dstate, s->spec_nf, s->d_spec_omega,
         s->d_spec_acc, s->d_spec_samples);
@@ -819,7 +821,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
       cudaEventRecord(s->ev_join, s->side);
       cudaStreamWaitEvent(s->stream, s->ev_join, 0);
     }
-    launch_scan(s, 1, s->cur);
+    k_advance<<<1, 1, 0, s->stream>>>(s->dstate, s->cur);
   }
   s->cur = 1 - s->cur;
   cudaError_t e = cudaGetLastError();

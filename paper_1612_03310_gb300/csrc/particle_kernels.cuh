@@ -875,6 +875,14 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_resort_small(
     perm[(long long)s_off[key[q]] + rank[q]] = (int)q;
 }
 
+// End of a step without particles: the step counter, and no source can be
+// nonzero any more (the update of level parity c cleared what it read, and
+// nothing deposits), so that the following updates skip the sources' loads.
+__global__ void k_advance(StepState* __restrict__ st, int c) {
+  st->n += 1;
+  st->src_all[c] = 0;
+}
+
 // Copy-out in the original particle order: FP64 positions from (cell, f).
 template <typename T, typename U>
 __global__ void k_copy_out(PicP<T> p, Parts<T, U> P, long long np, double* __restrict__ out) {

@@ -66,3 +66,24 @@ def test_resort_key_counts(M, orc, shape):  # noqa: F811
     g = inputs.random_grid(51, *shape)
     P = inputs.random_particles(52, g, 3000, u_scale=0.2)
     check(M, orc, g, dict(C1_UND, z_ent_lab=0.0), P, "P32_U64", (1, 4))
+
+
+def test_no_particles_sources_once(M, orc):  # noqa: F811
+    # without particles a set source drives one update, and the following
+    # updates read none
+    g = inputs.random_grid(61, 20, 18, 24)
+    src = 1e3 * np.random.default_rng(3).standard_normal((g["nz"], g["ny"], g["nx"]))
+    with M.Simulation(dict(g, boundary=1), None, None, precision=M.P64) as sim:
+        o = orc.OracleSim(g, None, dict(x=[], y=[], z=[], ux=[], uy=[], uz=[]))
+        for _ in range(2):
+            s = o.src.copy()
+            s[:o.n_cell] = src.ravel()
+            o.set_sources(s)
+            sim.set_field("Jx", src)
+            for n in (1, 6):
+                o.step(n)
+                sim.step(n)
+                sim.sync()
+                compare_fields(sim, o, 1e-10, names=["Ax", "Ex", "By", "Jx"])
+        assert sim.source_tiles() == (0, False)
+        assert sim.time()[0] == 14
