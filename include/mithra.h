@@ -387,11 +387,15 @@ mithra_status mithra_read_spectrum(mithra_sim* sim, double* dW_domega, int64_t* 
  *     neighbours read through L1; 1: the z-marching form, psi^n, D and source
  *     planes of a 32 x 8 column tile streamed through a shared-memory ring by
  *     TMA box loads (single-float levels only: MITHRA_P32, MITHRA_P64);
- *     2: register z-marching, a thread walks its column for lz planes with
- *     three planes' sums in registers.
+ *     2: z-marching in registers, a thread walks its column for lz planes with
+ *     three planes' sums in registers; in FP32, on grids (or in a batch) that
+ *     give every multiprocessor two CTAs of 8 planes in column tiles at least
+ *     0.7 full, with the planes brought to shared memory by TMA, lo parts
+ *     included, several in flight.
  *   lz: planes per CTA of the marching forms (0: about two waves of CTAs for
- *     variant 1; for variant 2 up to 16, fewer where the grid, or the batch
- *     the simulation is in, would leave multiprocessors without work).
+ *     variant 1; for variant 2 8 where the planes come by TMA, else up to 16,
+ *     fewer where the grid, or the batch the simulation is in, would leave
+ *     multiprocessors without work).
  *   push_variant 0: one thread per particle, E and B evaluated at the eight
  *     vertices from global memory; 1: persistent CTAs over 8^3-cell particle
  *     tiles with the potentials, E/B and the deposit block in shared memory.

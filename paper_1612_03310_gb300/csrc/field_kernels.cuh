@@ -785,6 +785,187 @@ __global__ void __launch_bounds__(kMX* kMY, (sizeof(T) == 4 ? 4 : 1)) k_potentia
   }
 }
 
+// Ring form of the FP32 update: the arithmetic of the register z-marching
+// form, with the level's planes (one vertex of halo; its lo parts two in x,
+// for the 16-byte start of their rows) and the increment's columns brought to
+// shared memory by TMA, kRStages planes in flight per CTA.  A thread's loads
+// then wait in shared memory instead of on DRAM and its addresses are 32-bit
+// constants, so that the compensated form too runs in 64 registers (four CTAs
+// an SM) and on packed FP32 pairs.  Sources come straight from global memory
+// in the tiles the particle step marked.  kMur: first-order Mur at the x
+// faces as in zloop_body.  Lo parts (kLo): none, by TMA, or by 8-byte cp.async
+// (odd nx: a row of lo parts then starts on 8 bytes, which TMA does not take).
+enum RingLo { kRingPlain = 0, kRingTma, kRingAsync };
+constexpr int kRX = 32, kRY = 8, kRStages = 4;
+constexpr int kRThreads = kRX * kRY;
+constexpr int kRPsi = (kRX + 2) * (kRY + 2) * 16;
+constexpr int kRLoX = kRX + 4;
+constexpr int kRLo = kRLoX * (kRY + 2) * 8;
+constexpr int kRD = kRThreads * 16;
+constexpr int kROffD = (kRPsi + 127) / 128 * 128;
+constexpr int kROffLo = kROffD + kRD;
+__host__ __device__ constexpr int ring_stage_bytes(int lo) {
+  return kROffLo + (lo ? (kRLo + 127) / 128 * 128 : 0);
+}
+__host__ __device__ constexpr int ring_smem_bytes(int lo) {
+  return kRStages * ring_stage_bytes(lo) + 2 * kRStages * 8;
+}
+
+template <int kLo, bool kMur>
+__global__ void __launch_bounds__(kRThreads, 4) k_potential_ring(
+    const __grid_constant__ CUtensorMap tm_cur, const __grid_constant__ CUtensorMap tm_lo,
+    const __grid_constant__ CUtensorMap tm_d, const __grid_constant__ StencilP<float> p,
+    const LoV4* __restrict__ curlo, V4<float>* __restrict__ nxt, LoV4* __restrict__ nxtlo,
+    V4<float>* __restrict__ D, V4<float>* __restrict__ src, int lz, int* __restrict__ err) {
+  typedef V4<float> F4;
+  constexpr int HX = kRX + 2, LX = kRLoX, kStage = ring_stage_bytes(kLo);
+  extern __shared__ __align__(128) unsigned char smem[];
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRStages * kStage);
+  uint64_t* empty = full + kRStages;
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int i0 = blockIdx.x * kRX, j0 = blockIdx.y * kRY;
+  const int i = i0 + tx, j = j0 + ty;
+  const int kb = max((int)blockIdx.z * lz, 1);
+  const int ke = min((int)blockIdx.z * lz + lz, p.nz - 1);
+  if (kb >= ke) return;             // uniform over the block
+  const int nplanes = ke - kb + 2;  // planes kb-1 .. ke of the level
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRStages; ++s) {
+      mbar_init(&full[s], kLo == kRingAsync ? 1 + kRThreads : 1);
+      mbar_init(&empty[s], kRThreads / 32);
+    }
+    mbar_fence_init();
+  }
+  __syncthreads();
+  // stage q holds the level's plane kb-1+q and, for updated planes, the
+  // increment of plane kb-2+q (the plane updated when stage q arrives)
+  auto issue = [&](int q) {
+    const int s = q % kRStages;
+    unsigned char* base = smem + s * kStage;
+    if (threadIdx.x == 0) {
+      const int kd = kb - 2 + q;
+      const bool cols = kd >= kb;
+      mbar_arrive_expect_tx(&full[s],
+                            kRPsi + (kLo == kRingTma ? kRLo : 0) + (cols ? kRD : 0));
+      tma_load_field(base, &tm_cur, i0 - 1, j0 - 1, kb - 1 + q, &full[s]);
+      if (kLo == kRingTma)
+        tma_load_field(base + kROffLo, &tm_lo, i0 - 2, j0 - 1, kb - 1 + q, &full[s]);
+      if (cols) tma_load_field(base + kROffD, &tm_d, i0, j0, kd, &full[s]);
+    }
+    if (kLo == kRingAsync) {
+      const LoV4* plane = curlo + (kb - 1 + q) * p.nxy;
+      for (int v = threadIdx.x; v < LX * (kRY + 2); v += kRThreads) {
+        const int ii = i0 - 2 + v % LX, jj = j0 - 1 + v / LX;
+        if (ii >= 0 && ii < p.nx && jj >= 0 && jj < p.ny)
+          cp_async<8>(reinterpret_cast<LoV4*>(base + kROffLo) + v, plane + jj * p.nx + ii);
+      }
+      cp_async_mbar_arrive(&full[s]);
+    }
+  };
+  for (int q = 0; q < kRStages && q < nplanes; ++q) issue(q);
+
+  const bool xb = kMur && (i == 0 || (i == p.nx - 1 && xhi_fused(p.nx)));
+  const bool active = j >= 1 && j <= p.ny - 2 && ((i >= 1 && i <= p.nx - 2) || xb);
+  const bool xwarp = kMur && __any_sync(0xffffffffu, xb && active);
+  const int from = i == 0 ? tx + 1 : (xb ? tx - 1 : tx);
+  const F4 zero = v4(0.0f, 0.0f, 0.0f, 0.0f);
+  // one plane's terms (plane_terms) from a stage
+  auto terms = [&](const unsigned char* base, F4* a, F4* b, F4* c, F4* cl) {
+    const F4* pl = reinterpret_cast<const F4*>(base) + (ty + 1) * HX + (tx + 1);
+    const F4 cc = pl[0];
+    F4 X = vadd<true>(vsub<true>(pl[1], cc), vsub<true>(pl[-1], cc));
+    F4 Y = vadd<true>(vsub<true>(pl[HX], cc), vsub<true>(pl[-HX], cc));
+    *cl = zero;
+    if (kLo) {
+      const LoV4* lo = reinterpret_cast<const LoV4*>(base + kROffLo) + (ty + 1) * LX + (tx + 2);
+      auto low = [&](int o) {
+        const LoV4 v = lo[o];
+        return v4_of(__bfloat1622float2(v.xy), __bfloat1622float2(v.zw));
+      };
+      const F4 ll = low(0);
+      X = vadd<true>(X, vadd<true>(vsub<true>(low(1), ll), vsub<true>(low(-1), ll)));
+      Y = vadd<true>(Y, vadd<true>(vsub<true>(low(LX), ll), vsub<true>(low(-LX), ll)));
+      *cl = ll;
+    }
+    *a = vfma<true>(p.rxA, X, vmul<true>(p.ryA, Y));
+    *b = vfma<true>(p.rxB, X, vmul<true>(p.ryB, Y));
+    *c = cc;
+  };
+  auto wait = [&](int q) {
+    mbar_wait_bounded(&full[q % kRStages], (uint32_t)((q / kRStages) & 1), err);
+    return smem + (q % kRStages) * kStage;
+  };
+  // each warp marks a stage it has read on the stage's empty barrier
+  auto release = [&](int q) {
+    __syncwarp();
+    if (tx == 0) mbar_arrive(&empty[q % kRStages]);
+  };
+  // refills the slot of stage q once every warp has read it: called a plane
+  // later, when they all have, or nearly
+  auto refill = [&](int q) {
+    if (q + kRStages >= nplanes) return;
+    if (kLo == kRingAsync || threadIdx.x == 0) {
+      mbar_wait_bounded(&empty[q % kRStages], (uint32_t)((q / kRStages) & 1), err);
+      if (threadIdx.x == 0) fence_proxy_async_smem();
+      issue(q + kRStages);
+    }
+  };
+  F4 ab, a0, cm, clm, c0, cl0;
+  {
+    F4 am, bm, b0;
+    terms(wait(0), &am, &bm, &cm, &clm);
+    release(0);
+    terms(wait(1), &a0, &b0, &c0, &cl0);
+    release(1);
+    refill(0);
+    ab = vadd<true>(am, b0);
+  }
+  const bool src_every = p.dirty == nullptr || *p.src_all != 0;
+  const int trow = (j >> 3) * p.ntx + (i >> 3), ntxy = p.ntx * p.nty;
+  long long c = (long long)kb * p.nxy + (long long)j * p.nx + i;
+  for (int k = kb; k < ke; ++k, c += p.nxy) {
+    const int q = k - kb + 2;
+    const unsigned char* base = wait(q);
+    F4 ap, bp, cp, clp;
+    terms(base, &ap, &bp, &cp, &clp);
+    const F4 dm = reinterpret_cast<const F4*>(base + kROffD)[threadIdx.x];
+    F4 L = vfma<true>(p.rz2, vadd<true>(vsub<true>(cp, c0), vsub<true>(cm, c0)),
+                      vadd<true>(ab, ap));
+    if (kLo) L = vfma<true>(p.rz2, vadd<true>(vsub<true>(clp, cl0), vsub<true>(clm, cl0)), L);
+    release(q);
+    refill(q - 1);
+    F4 sv = zero;
+    if (active && (src_every || p.dirty[(k >> 3) * ntxy + trow] != 0)) sv = src[c];
+    F4 dp = next_increment<true>(p, dm, L, sv);
+    if (kMur && xwarp) {  // warp-uniform
+      const F4 dq = v4(__shfl_sync(0xffffffffu, dp.x, from), __shfl_sync(0xffffffffu, dp.y, from),
+                       __shfl_sync(0xffffffffu, dp.z, from), __shfl_sync(0xffffffffu, dp.w, from));
+      const F4 mq = v4(__shfl_sync(0xffffffffu, dm.x, from), __shfl_sync(0xffffffffu, dm.y, from),
+                       __shfl_sync(0xffffffffu, dm.z, from), __shfl_sync(0xffffffffu, dm.w, from));
+      if (xb) dp = mur_beta0(p, 1) * (dq - dm) + mq;
+    }
+    if (!p.space_charge) dp.w = 0.0f;
+    if (active) {
+      if (nonzero(sv)) src[c] = zero;
+      D[c] = dp;
+      const F4 s = vadd<true>(c0, dp);
+      if (kLo) {  // comp_add on pairs
+        const F4 bb = vsub<true>(s, c0);
+        const F4 e = vadd<true>(vsub<true>(c0, vsub<true>(s, bb)), vsub<true>(dp, bb));
+        const F4 l = vadd<true>(cl0, e);
+        const F4 h = vadd<true>(s, l);
+        nxt[c] = h;
+        st_lo(nxtlo, c, vsub<true>(l, vsub<true>(h, s)));
+      } else {
+        nxt[c] = s;
+      }
+    }
+    ab = vadd<true>(a0, bp);
+    a0 = ap;
+    cm = c0; clm = cl0; c0 = cp; cl0 = clp;
+  }
+}
+
 // E and B at vertex v (interior) at t = (n+1/2) dt from psi^{n+1} (pn) and
 // the increment D = psi^{n+1} - psi^n:  B = (curl A^n + curl A^{n+1}) / 2 is
 // the curl of the mid level pn - D/2; E = -D_A / dt - grad phi^n with

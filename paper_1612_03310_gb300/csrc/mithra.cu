@@ -126,6 +126,8 @@ struct mithra_sim {
   CUtensorMap tm_box_d;   // increment, 11^3 boxes
   CUtensorMap tm_col_d;   // increment, 32 x 8 column boxes of the marching update
   CUtensorMap tm_col_s;   // sources, 32 x 8 column boxes
+  CUtensorMap tm_lo[2];   // lo parts, plane boxes of the ring update
+  bool have_lo_map = false;  // tm_lo is set (compensated levels, even nx)
   int push_variant = 0;   // 0 per-particle, 1 tiled (needs the box maps)
   int push_grid = 0;      // persistent CTAs of the tiled particle step
   int push_max_per_sm = 1;
@@ -453,6 +455,31 @@ int plane_run(const mithra_sim* s) {
   return lz;
 }
 
+// Planes per CTA of the ring form of the FP32 update (k_potential_ring), 0: the
+// register form.  The ring form takes grids (or batches) that give every
+// multiprocessor two CTAs of 8 planes, in column tiles at least 0.7 full (its
+// CTAs do whole tiles, the register form's idle warps leave).  Potential
+// scope, register and ring form: 128 x 128 x 1024 cells compensated 276 and
+// 230 us, plain 193 and 185; 256 x 256 x 2048 compensated 1961 and 1661; 101 x
+// 75 x 413 93 and 83; 64 x 64 x 256 29 and 27; but 32 x 32 x 128 16 and 20, 65
+// x 65 x 256 31 and 39.  Runs of 4, 16 and 64 planes took 246, 235 and 262 us
+// of the first: longer ones part in z from the CTAs that share their halo.
+int ring_run(const mithra_sim* s) {
+  if (s->prec == MITHRA_P64 || !s->have_tm || s->stencil_variant != 2) return 0;
+  const int cols = (s->g.nx + 31) / 32 * 32, rows = (s->g.ny + 7) / 8 * 8;
+  if (10LL * s->g.nx * s->g.ny < 7LL * cols * rows) return 0;
+  int64_t np = 0, planes = column_planes(s->g);
+  if (s->in_batch) batch_totals(s->in_batch, &np, &planes);
+  if (planes < 8LL * 2 * s->n_sm) return 0;
+  return s->lz_auto ? 8 : s->lz;
+}
+
+// Planes per CTA that the single simulation's z-marching update takes.
+int effective_run(const mithra_sim* s) {
+  const int ring = ring_run(s);
+  return ring > 0 ? ring : plane_run(s);
+}
+
 // Tiles below this many particles take the sparse path (0: none): the
 // caller's threshold, or 32 (FP64: 64) on grids of many tiles per CTA, where
 // the staged path's time is its number of tiles (128 x 128 x 1024 cells, 2^21
@@ -541,6 +568,13 @@ int default_lz(const mithra_grid* g, int resident) {
 
 template <typename T>
 mithra_status setup_march(mithra_sim* s) {
+  if constexpr (sizeof(T) == 4) {
+    for (auto kern : {k_potential_ring<kRingPlain, true>, k_potential_ring<kRingPlain, false>,
+                      k_potential_ring<kRingTma, true>, k_potential_ring<kRingTma, false>,
+                      k_potential_ring<kRingAsync, true>, k_potential_ring<kRingAsync, false>})
+      MCHECK(s, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     ring_smem_bytes(kRingTma)));
+  }
   MCHECK(s, cudaFuncSetAttribute(k_potential_march<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  march_smem_bytes<T>()));
   int dev = 0, nsm = 0, per_sm = 0;
@@ -655,7 +689,26 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
       const int lz = plane_run(s);
       dim3 blk(32, 8, 1);
       dim3 grd((s->g.nx + 31) / 32, (s->g.ny + 7) / 8, (s->g.nz + lz - 1) / lz);
-      if (L0 && fused)
+      const int rl = ring_run(s);
+      if constexpr (sizeof(T) == 4) {
+        if (rl > 0) {
+          const int lo = !L0 ? kRingPlain : (s->have_lo_map ? kRingTma : kRingAsync);
+          auto kern = lo == kRingPlain
+                          ? (fused ? k_potential_ring<kRingPlain, true>
+                                   : k_potential_ring<kRingPlain, false>)
+                      : lo == kRingTma ? (fused ? k_potential_ring<kRingTma, true>
+                                                : k_potential_ring<kRingTma, false>)
+                                       : (fused ? k_potential_ring<kRingAsync, true>
+                                                : k_potential_ring<kRingAsync, false>);
+          grd.z = (s->g.nz + rl - 1) / rl;
+          kern<<<grd, kRThreads, ring_smem_bytes(lo), s->stream>>>(
+              s->tm[s->cur], s->tm_lo[s->cur], s->tm_col_d, sp, L0, P1, L1, Dn, S, rl,
+              &s->dstate->err);
+        }
+      }
+      if (rl > 0) {
+        // launched above
+      } else if (L0 && fused)
         k_potential_zloop_mur1<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else if (L0)
         k_potential_zloop<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
@@ -1219,6 +1272,11 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
                                   kTP) &&
                  encode_field_map(&s->tm_col_d, s->D, es, grid->nx, grid->ny, grid->nz, kMX, kMY) &&
                  encode_field_map(&s->tm_col_s, s->S, es, grid->nx, grid->ny, grid->nz, kMX, kMY);
+    s->have_lo_map = s->have_tm && s->PL[0] &&
+                   encode_lo_map(&s->tm_lo[0], s->PL[0], grid->nx, grid->ny, grid->nz, kRLoX,
+                                 kRY + 2) &&
+                   encode_lo_map(&s->tm_lo[1], s->PL[1], grid->nx, grid->ny, grid->nz, kRLoX,
+                                 kRY + 2);
     // defaults: the register z-marching update (fastest on every grid the
     // autotuner has timed, any precision) and the tiled push when TMA maps
     // exist
@@ -1229,7 +1287,7 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
       mithra_status r = setup_push_grid<T, U>(s);
       return r == MITHRA_OK ? setup_march<T>(s) : r;
     });
-    s->lz = plane_run(s);
+    s->lz = effective_run(s);
     if (st != MITHRA_OK) {
       std::string msg = s->err;
       return bail(st, msg);
@@ -1742,7 +1800,7 @@ mithra_status mithra_set_tuning(mithra_sim* s, const mithra_tuning* t) {
   // (the run mithra_get_tuning showed, set again, stays the library's choice)
   s->lz_auto = t->stencil_variant == 2 && (t->lz == 0 || (s->lz_auto && t->lz == s->lz));
   s->lz = t->lz > 0 ? t->lz
-                    : (s->lz_auto ? plane_run(s) : default_lz(&s->g, s->march_resident));
+                    : (s->lz_auto ? effective_run(s) : default_lz(&s->g, s->march_resident));
   s->push_variant = t->push_variant;
   s->push_ctas_per_sm = t->push_ctas_per_sm;
   s->push_sparse_below = t->push_sparse_below;

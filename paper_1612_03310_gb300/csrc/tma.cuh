@@ -68,6 +68,13 @@ __device__ inline void cp_async(void* dst, const void* src) {
 __device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ inline void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
+// arrives on bar (one of its expected arrivals) when this thread's earlier
+// cp.async copies have landed
+__device__ inline void cp_async_mbar_arrive(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_addr(bar))
+               : "memory");
+}
+
 __device__ inline void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -128,6 +135,24 @@ inline bool encode_field_map(CUtensorMap* tm, void* base, int elem_bytes, int nx
                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+// Tensor map of the lo parts of a compensated level (4 bfloat16, 8 bytes, a
+// vertex), folded as in encode_field_map; load_field's element 4 i is then a
+// multiple of 16 bytes for even i only.  Fails for odd nx (rows must start on
+// 16 bytes).
+inline bool encode_lo_map(CUtensorMap* tm, void* base, int nx, int ny, int nz, int bx, int by) {
+  TensorMapEncodeTiled enc = tensor_map_encoder();
+  if (!enc || (nx & 1)) return false;
+  const cuuint64_t row = 8ull * nx;
+  const cuuint64_t dims[3] = {4ull * nx, (cuuint64_t)ny, (cuuint64_t)nz};
+  const cuuint64_t strides[2] = {row, row * ny};
+  const cuuint32_t box[3] = {4u * bx, (cuuint32_t)by, 1u};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+         CUDA_SUCCESS;
 }
 
 }  // namespace mithra

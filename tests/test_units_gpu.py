@@ -1,4 +1,5 @@
-"""The particle step's work units and the one-kernel re-sort, at the sizes
+"""The particle step's work units, the one-kernel re-sort and the ring form of
+the potential update, at the sizes
 where they can go wrong: tiles of exactly one, a whole number and one more
 than a whole number of units, key counts around the scans' block sizes, the
 sparse tiles' kernel beside the units, an empty bunch; against the oracle."""
@@ -6,7 +7,8 @@ import numpy as np
 import pytest
 
 from paper_1612_03310_gb300 import inputs
-from test_parity_gpu import C1_UND, M, compare_fields, compare_particles  # noqa: F401
+from test_parity_gpu import (C1_UND, M, compare_fields, compare_particles,  # noqa: F401
+                             oracle_fields, set_state)
 
 pytestmark = pytest.mark.gpu
 
@@ -87,3 +89,29 @@ def test_no_particles_sources_once(M, orc):  # noqa: F811
                 compare_fields(sim, o, 1e-10, names=["Ax", "Ex", "By", "Jx"])
         assert sim.source_tiles() == (0, False)
         assert sim.time()[0] == 14
+
+
+@pytest.mark.parametrize("prec", ["P32", "P32_C"])
+@pytest.mark.parametrize("boundary", [1, 2])
+@pytest.mark.parametrize("shape", [(64, 72, 273), (129, 40, 155), (130, 48, 155), (97, 80, 243),
+                                   (127, 57, 155)])
+def test_ring_update(M, orc, prec, boundary, shape):  # noqa: F811
+    # the ring form of the update (grids of at least two 8-plane column tiles
+    # a multiprocessor): odd nx (lo parts by cp.async) and even (by TMA), nx a
+    # multiple of 32, one more (the x+ face in the boundary kernel) and one
+    # less, last tiles of one row or plane, runs that end in a short one; a
+    # level with everything random so that every face is seen
+    g = dict(inputs.random_grid(71, *shape), boundary=boundary)
+    f = inputs.random_fields(72, g, scale=1e-9)
+    f = {k: v.astype(np.float32).astype(np.float64) for k, v in f.items()}
+    P = inputs.random_particles(73, g, 500, u_scale=0.2)
+    o = orc.OracleSim(g, None, P)
+    with M.Simulation(g, None, P, precision=getattr(M, prec)) as sim:
+        set_state(sim, o, f)
+        o.step(2)
+        sim.step(2)
+        sim.sync()
+        compare_fields(sim, o, 1e-5)
+        for nm in ("Ax", "Az", "phi"):  # the largest vertex too, of the largest value
+            ref = oracle_fields(o)[nm]
+            assert np.abs(sim.copy_field(nm) - ref).max() <= 1e-5 * np.abs(ref).max(), nm
