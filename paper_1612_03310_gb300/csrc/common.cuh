@@ -188,6 +188,7 @@ struct StencilP {
   int nx, ny, nz;
   long long nxy;
   T rxA, rxB, ryA, ryB, rz2;  // rx^2 A, rx^2 (1 - 2A), ry^2 A, ry^2 (1 - 2A), rz^2
+  T kap;                      // (1 - 2A) / A (A > 0)
   T sA, sphi;                 // (c dt)^2 mu0 and (c dt)^2 / eps0
   T mb0[8];
   // second-order Mur on face vertices (mur2 != 0): m2[a][0], m2[a][1] =

@@ -294,6 +294,7 @@ StencilP<T> make_stencil(const mithra_grid& g) {
   p.ryA = (T)(ry2 * A);
   p.ryB = (T)(ry2 * (1.0 - 2.0 * A));
   p.rz2 = (T)rz2;
+  p.kap = (T)(A > 0.0 ? (1.0 - 2.0 * A) / A : 1.0);
   p.sA = (T)(cdt * cdt * kMu0);
   p.sphi = (T)(cdt * cdt / kEps0);
   for (int m = 0; m < 8; ++m) {
