@@ -13,16 +13,15 @@
 //      (Eq. fieldInterpolation), rest-frame undulator field, Boris
 //      (Eq. BorisScheme; 1/gamma to the particle precision's rounding, by a
 //      float-float Newton step in the FP32 forms), cell carry;
-//   4. deposits rho^{n+3/2} (end point) into a shared-memory block over the
-//      11^3 vertices -- in the FP32 forms as exact int32 fixed-point sums,
-//      added to the global sources once per touched vertex -- and
-//      J^{n+1} (mid point) with FP32 vector atomics straight into L2 (FP64:
-//      both components through a shared FP64 block).
+//   4. deposits rho^{n+3/2} (end point) and J^{n+1} (mid point) with atomics
+//      straight into L2 (FP32 vector atomics for J), in the FP32 forms rho
+//      through a shared-memory block over the 11^3 vertices as exact int32
+//      fixed-point sums, added to the global sources once per touched vertex.
 // A particle whose sub-step leaves the tile (n_sub > 1) gathers from global
 // memory, and one whose deposit leaves the 11^3 block deposits with global
 // atomics: the same arithmetic on another path.  Sparse tiles (fewer
-// particles than the staging pays for) are then taken one per warp on that
-// global path.  Particles lost in earlier steps are only moved to the
+// particles than the staging pays for) are taken one per warp on that global
+// path by a kernel of their own (k_push_sparse), beside this one.  Particles lost in earlier steps are only moved to the
 // other buffer and keep their re-sort bucket.
 #pragma once
 #include "common.cuh"
@@ -100,38 +99,6 @@ __device__ inline void eb_local(const PicP<T>& p, const V4<T>* __restrict__ sP,
   B = v4(b[0], b[1], b[2], (T)0);
 }
 
-// CIC deposit into the shared 11^3 block whose vertex (0,0,0) is global
-// (i0-1, j0-1, k0-1), one array per component (stride kTPC: J_x, J_y, J_z,
-// rho); kRho selects the charge (one component) or the current (three).
-// Falls back to global atomics outside the block.
-template <bool kRho, typename T>
-__device__ inline void deposit_tile(const PicP<T>& p, T* __restrict__ sJ,
-                                    V4<T>* __restrict__ src, int i0, int j0, int k0, int i, int j,
-                                    int k, T fx, T fy, T fz, T jx, T jy, T jz, T rho) {
-  const int li = i - (i0 - 1), lj = j - (j0 - 1), lk = k - (k0 - 1);
-  if (li < 0 || li > kTP - 2 || lj < 0 || lj > kTP - 2 || lk < 0 || lk > kTP - 2) {
-    deposit_cic(p, src, i, j, k, fx, fy, fz, jx, jy, jz, rho);
-    return;
-  }
-  const T wx[2] = {(T)1 - fx, fx}, wy[2] = {(T)1 - fy, fy}, wz[2] = {(T)1 - fz, fz};
-#pragma unroll
-  for (int K = 0; K < 2; ++K)
-#pragma unroll
-    for (int J = 0; J < 2; ++J)
-#pragma unroll
-      for (int I = 0; I < 2; ++I) {
-        const T w = wx[I] * wy[J] * wz[K];
-        T* a = sJ + ((lk + K) * kTP + (lj + J)) * kTP + (li + I);
-        if (kRho) {
-          atomicAdd(a + 3 * kTPC, w * rho);
-        } else {
-          atomicAdd(a, w * jx);
-          atomicAdd(a + kTPC, w * jy);
-          atomicAdd(a + 2 * kTPC, w * jz);
-        }
-      }
-}
-
 // Charge deposit of the FP32 forms into the 11^3 block.  Every rho
 // contribution is w q/V with a CIC weight w in [0, 1], so the block sums the
 // integers hi = rint(w 2^b) and lo = rint((w 2^b - hi) 2^b) with int32
@@ -159,7 +126,7 @@ __device__ inline void deposit_rho_fixed(const PicP<T>& p, int* __restrict__ hi,
   const int li = i - (i0 - 1), lj = j - (j0 - 1), lk = k - (k0 - 1);
   if (li < 0 || li > kTP - 2 || lj < 0 || lj > kTP - 2 || lk < 0 ||
       lk > kTP - 2) {
-    deposit_cic(p, src, i, j, k, fx, fy, fz, (T)0, (T)0, (T)0, p.qV);
+    deposit_rho(p, src, i, j, k, fx, fy, fz, p.qV);
     return;
   }
   const float wx[2] = {1.0f - (float)fx, (float)fx}, wy[2] = {1.0f - (float)fy, (float)fy},
@@ -317,11 +284,12 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   V2<T>* sB = reinterpret_cast<V2<T>*>(smem + tile_b2_offset<T>());   // B_y, B_z
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + tile_bar_offset<T>());
   static_assert(tile_slot_bytes<T, U>() <= tile_box_bytes<T>(), "slots fit the increment box");
-  // deposit block, reuses the psi box once E, B are built.  FP64: one array
-  // per component (J_x, J_y, J_z, rho), so that atomics of a component from
-  // different vertices spread over all banks.  FP32: the fixed-point rho
-  // sums (hi, lo), the current going to global memory directly (vector
-  // atomics in L2, measured faster than FP32 shared-memory atomics).
+  // deposit block of the FP32 forms, reuses the psi box once E, B are built:
+  // the fixed-point rho sums (hi, lo).  The current goes to global memory
+  // directly (vector atomics in L2, measured faster than FP32 shared-memory
+  // atomics), and in FP64 the charge too: shared FP64 atomics are
+  // compare-and-swap loops (96 x 80 x 384 cells, 4e5 particles: 482 us with
+  // both in shared memory, 467 with the charge there, 458 without).
   constexpr bool kF32 = sizeof(T) == 4;
   // this thread's next-particle slot (stride kPushThreads between the
   // components), in
@@ -337,7 +305,6 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
                                                       3 * (int)sizeof(U))) +
                threadIdx.x;
   int* sl_pos = sl_id + kPushThreads;
-  T* sJ = reinterpret_cast<T*>(sP);
   int* sRh = reinterpret_cast<int*>(sP);
   int* sRl = sRh + kTPC;
   __shared__ int s_tile;
@@ -455,8 +422,6 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
         bsh = min(21, 30 - (nt > 1 ? 32 - __clz(nt - 1) : 0));
         sb = __int_as_float((127 + bsh) << 23);
         for (int c = tid; c < 2 * kTPC; c += blockDim.x) sRh[c] = 0;
-      } else {
-        for (int c = tid; c < 4 * kTPC; c += blockDim.x) sJ[c] = (T)0;
       }
       __syncthreads();
 
@@ -493,18 +458,12 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
             },
             [&](bool rho, int i, int j, int k, const T* f, T jx, T jy, T jz, T q) {
               far_deposit(a, i0, j0, k0, i, j, k);
-              if (kF32) {
-                if (rho)
-                  deposit_rho_fixed(p, sRh, sRl, src, i0, j0, k0, i, j, k, f[0], f[1], f[2], sb);
-                else
-                  deposit_cic(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz, (T)0);
-              } else if (rho) {
-                deposit_tile<true>(p, sJ, src, i0, j0, k0, i, j, k, f[0], f[1], f[2], jx, jy, jz,
-                                   q);
-              } else {
-                deposit_tile<false>(p, sJ, src, i0, j0, k0, i, j, k, f[0], f[1], f[2], jx, jy, jz,
-                                    q);
-              }
+              if (!rho)
+                deposit_j(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz);
+              else if constexpr (kF32)
+                deposit_rho_fixed(p, sRh, sRl, src, i0, j0, k0, i, j, k, f[0], f[1], f[2], sb);
+              else
+                deposit_rho(p, src, i, j, k, f[0], f[1], f[2], q);
             },
             [&]() { return *sl_cell; },
             [&](T* f, U* u) {
@@ -528,15 +487,6 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
             const int a = c % kTP, b = (c / kTP) % kTP, cc = c / (kTP * kTP);
             atomicAdd(&src[cidx(i0 - 1 + a, j0 - 1 + b, k0 - 1 + cc, p.nx, p.nxy)].w,
                       (T)((float)h * s1 + (float)l * s2));
-          }
-        }
-      } else {
-        for (int c = tid; c < kTPC; c += blockDim.x) {
-          const V4<T> v = v4(sJ[c], sJ[kTPC + c], sJ[2 * kTPC + c], sJ[3 * kTPC + c]);
-          if (v.x != (T)0 || v.y != (T)0 || v.z != (T)0 || v.w != (T)0) {
-            const int a = c % kTP, b = (c / kTP) % kTP, cc = c / (kTP * kTP);
-            dep_add(src + cidx(i0 - 1 + a, j0 - 1 + b, k0 - 1 + cc, p.nx, p.nxy), v.x, v.y, v.z,
-                    v.w);
           }
         }
       }
@@ -620,7 +570,10 @@ __device__ inline void push_sparse_tile(const PushArgs<T, U>& a, int tile, doubl
         },
         [&](bool rho, int i, int j, int k, const T* f, T jx, T jy, T jz, T q) {
           far_deposit(a, i0, j0, k0, i, j, k);
-          deposit_cic(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz, q);
+          if (rho)
+            deposit_rho(p, src, i, j, k, f[0], f[1], f[2], q);
+          else
+            deposit_j(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz);
         },
         [&]() { return P.cell[pos]; },
         [&](T* f, U* u) {

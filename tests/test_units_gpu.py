@@ -115,3 +115,26 @@ def test_ring_update(M, orc, prec, boundary, shape):  # noqa: F811
         for nm in ("Ax", "Az", "phi"):  # the largest vertex too, of the largest value
             ref = oracle_fields(o)[nm]
             assert np.abs(sim.copy_field(nm) - ref).max() <= 1e-5 * np.abs(ref).max(), nm
+
+
+def test_fp64_moves_across_cells(M, orc):  # noqa: F811
+    # the FP64 cell carry: fractions 0 and just below 1, steps that end on a
+    # face, before it and past it along each axis
+    g = inputs.random_grid(81, 24, 24, 24)
+    h = np.array([g["dx"], g["dy"], g["dz"]])
+    r0 = np.array([g["x0"], g["y0"], g["z0"]])
+    frac = [0.0, 1e-18, 0.25, 0.5, 1.0 - 2.0 ** -40]
+    pos, mom = [], []
+    for f in frac:
+        for a in range(3):
+            for u in (-3.0, -1e-3, 0.0, 1e-3, 3.0):
+                p = np.full(3, 10.5)
+                p[a] = 10.0 + f
+                v = np.zeros(3)
+                v[a] = u
+                pos.append(r0 + p * h)
+                mom.append(v)
+    pos, mom = np.array(pos), np.array(mom)
+    P = dict(x=pos[:, 0], y=pos[:, 1], z=pos[:, 2], ux=mom[:, 0], uy=mom[:, 1], uz=mom[:, 2],
+             q_macro=-1e-18)
+    check(M, orc, g, None, P, "P64", (1, 1, 3))
