@@ -133,6 +133,9 @@ struct mithra_sim {
   int push_max_per_sm = 1;
   int push_ctas_per_sm = 0;
   int push_sparse_below = 0;  // tiles with fewer particles take the per-warp path
+  // threshold of the scan that built the lists in use (they may hold sparse
+  // tiles after the threshold has changed to none)
+  int list_below = 0;
   int n_sm = 152;
   mithra_batch* in_batch = nullptr;  // the batch that steps this sim, if any
   // per-kernel event timing
@@ -494,6 +497,10 @@ int sparse_below(const mithra_sim* s) {
   return s->prec == MITHRA_P64 ? 64 : 32;
 }
 
+// Whether a step's lists can hold sparse tiles: the lists in use at the
+// launch or capture, or those of the re-sorts that follow.
+bool may_be_sparse(const mithra_sim* s) { return s->list_below > 0 || sparse_below(s) > 0; }
+
 // Blocks of the sparse tiles' kernel: eight a multiprocessor (32 warps), so
 // that the device takes some 5000 sparse tiles at once.
 unsigned sparse_grid(int n_sm) { return 8u * n_sm; }
@@ -506,7 +513,7 @@ void launch_scan(mithra_sim* s, int advance, int parity, cudaStream_t q = nullpt
   int* const cnt = s->count[parity];
   int* const next = s->count[1 - parity];
   const int nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
-  const int below = sparse_below(s);
+  const int below = s->list_below = sparse_below(s);
   const int chunk = unit_chunk(particles_beside(s), s->push_grid);
   k_scan_partials<kRestored><<<nb, kScanBlock, 0, q>>>(cnt, s->offset, s->nkeys,
                                                        below, chunk, s->scan_part);
@@ -617,13 +624,14 @@ bool small_resort(const mithra_sim* s) { return s->count[0] != s->count[1]; }
 // grids of few tiles.
 void launch_resort(mithra_sim* s, int parity, cudaStream_t q) {
   if (small_resort(s)) {
+    s->list_below = sparse_below(s);
     // the scan's scope holds the whole re-sort, the slot map's is empty
     { ProfScope none(s, K_SLOT_MAP); }
     ProfScope ps(s, K_SCAN);
     const unsigned nb = std::min<unsigned>(blocks_for(s->np, 4 * kSmallThreads), 2 * s->n_sm);
     k_resort_small<<<nb, kSmallThreads, 0, q>>>(
         s->count[parity], s->count[1 - parity], s->offset, s->tiles, s->units, s->nkeys,
-        sparse_below(s), unit_chunk(particles_beside(s), s->push_grid), s->dstate, s->np, s->key,
+        s->list_below, unit_chunk(particles_beside(s), s->push_grid), s->dstate, s->np, s->key,
         s->rank, s->perm);
     return;
   }
@@ -752,7 +760,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
   // the sparse tiles' kernel and the plane diagnostics run beside the tiled
   // particle step; with per-kernel timing every kernel stays on the
   // simulation's stream
-  const bool sparse = s->np > 0 && s->push_variant == 1 && s->have_tm && sparse_below(s) > 0;
+  const bool sparse = s->np > 0 && s->push_variant == 1 && s->have_tm && may_be_sparse(s);
   const bool branch = !s->profiling && (s->power_cap > 0 || s->spec_nf > 0 || sparse);
   cudaStream_t dq = s->stream;
   if (branch) {
@@ -2205,7 +2213,10 @@ mithra_status capture_fused_typed(mithra_batch* b) {
                      : (lo ? k_push_sparse<false, T, U, kAnyLo, true>
                            : k_push_sparse<false, T, U, false, true>);
   bool sparse = false;
-  for (const BatchMember<T, U>& m : tab) sparse = sparse || m.sparse_below > 0;
+  for (mithra_sim* s : b->sims) {
+    sparse = sparse || may_be_sparse(s);
+    s->list_below = sparse_below(s);  // the captured scans'
+  }
   if (cudaFuncSetAttribute(kpush, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
       cudaSuccess)
     return bfail(b, MITHRA_ECUDA, "batched particle step: shared memory attribute");

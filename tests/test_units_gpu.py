@@ -138,3 +138,28 @@ def test_fp64_moves_across_cells(M, orc):  # noqa: F811
     P = dict(x=pos[:, 0], y=pos[:, 1], z=pos[:, 2], ux=mom[:, 0], uy=mom[:, 1], uz=mom[:, 2],
              q_macro=-1e-18)
     check(M, orc, g, None, P, "P64", (1, 1, 3))
+
+
+@pytest.mark.parametrize("fused", [None, True, False])
+def test_sparse_threshold_switched_off(M, orc, fused):  # noqa: F811
+    # lists built with every tile sparse, then a threshold of none: the step
+    # that still runs on those lists pushes their tiles too
+    g = inputs.random_grid(91, 32, 24, 24)
+    P = inputs.random_particles(92, g, 2000, u_scale=0.2)
+    und = dict(C1_UND, z_ent_lab=0.0)
+    o = orc.OracleSim(g, und, P)
+    with M.Simulation(dict(g, boundary=1), und, P, precision=M.P32_U64) as sim, M.Batch() as b:
+        for below, n in ((1 << 30, 4), (0, 4), (1 << 30, 3), (1, 2)):
+            sim.set_tuning(push_sparse_below=below)
+            if fused is not None:
+                b.set_mode(fused)
+                b.add(sim)
+                b.step(n)
+                b.sync()
+                b.remove(sim)
+            else:
+                sim.step(n)
+            o.step(n)
+            sim.sync()
+            compare_fields(sim, o, 1e-5, names=["Ex", "Bz", "phi", "Jx", "rho"])
+            compare_particles(sim, o, 2e-5, 1e-5)
