@@ -466,15 +466,16 @@ mithra_status mithra_plane_power_noalloc(const mithra_grid* grid, double gamma0,
  * member simulations together, two steps per replay of one captured CUDA
  * graph (two steps return each member's ping-pong buffers to their state at
  * capture).  Two forms of the graph:
- *   - fused: a step is eight launches whatever the number of members (for
- *     every 30 members of the particle step and 96 of the grid phases one
- *     more): the boundary rest, the potential update, the power sample, the
- *     numbering of the members' tiles, the particle step, the two scan
- *     passes of the re-sort and its slot map, each one kernel over a work list
- *     that spans all members (flat block lists for the grid phases,
- *     persistent CTAs taking every member's tiles from one counter for the
- *     particle step), with each member's arguments in the launch's
- *     parameter space or a device table.  The members must share the
+ *   - fused: a step is a handful of launches whatever the number of members
+ *     (for every 30 members of the particle step, beside each other, and 96
+ *     of the grid phases one more): the boundary rest, the potential update,
+ *     the power sample, the numbering of the members' work units, the
+ *     particle step, and the re-sort (one kernel where every member has at
+ *     most 4096 tiles, else two scan passes and the slot map), each over a
+ *     work list that spans all members (flat block lists for the grid phases,
+ *     persistent CTAs taking every member's units from one counter for the
+ *     particle step), with each member's arguments in the launch's parameter
+ *     space or a device table.  The members must share the
  *     precision form, undulator type and boundary order, use the register
  *     z-marching update and the tiled particle step, and record no seed,
  *     spectrum or bunch samples;

@@ -22,6 +22,7 @@
 
 namespace mithra {
 
+// kBPSlot: the slot map's blocks, or the whole re-sort's of small members
 enum BatchPhase { kBPMur = 0, kBPZ, kBPPow, kBPScan, kBPSlot, kBPCount };
 
 // Member of flat block g: the m with blk[m] <= g < blk[m+1] (blk has M + 1
@@ -148,30 +149,32 @@ __global__ void __launch_bounds__(256) kb_power(const BatchMember<T, U>* __restr
 // counter (k_push_sparse strides over their sparse tiles); kb_tile_prefix
 // numbers both member after member (from the lists the last re-sort left)
 // and clears the counter.
+// One block a group of kPushGroup members, whose part of `prefs` holds Mg + 1
+// entries of each prefix, then the counter (prefs_of).
+__host__ __device__ inline int* prefs_of(int* prefs, int group) {
+  return prefs + 2 * group * kPushGroup + 3 * group;
+}
 template <typename T, typename U>
-__global__ void __launch_bounds__(1024) kb_tile_prefix(const BatchMember<T, U>* __restrict__ mem,
-                                                       int M, int* __restrict__ pref,
-                                                       int* __restrict__ spref,
-                                                       int* __restrict__ work) {
-  __shared__ Pair ws[32];
-  Pair base = 0;
-  for (int c0 = 0; c0 < M; c0 += blockDim.x) {
-    const int m = c0 + threadIdx.x;
-    Pair n = 0;
-    if (m < M) n = pair_of(mem[m].units[0].x, mem[m].st->n_sparse);
-    Pair tot;
-    const Pair ex = base + block_exclusive_scan(n, ws, &tot);
-    if (m < M) {
-      pref[m] = pair_lo(ex);
-      spref[m] = pair_hi(ex);
-    }
-    base += tot;
-    __syncthreads();
+__global__ void __launch_bounds__(32) kb_tile_prefix(const BatchMember<T, U>* __restrict__ mem,
+                                                     int M, int* __restrict__ prefs) {
+  static_assert(kPushGroup <= 32, "a warp scans a group");
+  const int g0 = blockIdx.x * kPushGroup, Mg = min(kPushGroup, M - g0);
+  int* pref = prefs_of(prefs, blockIdx.x);
+  int* spref = pref + Mg + 1;
+  const int m = threadIdx.x;
+  Pair v = 0;
+  if (m < Mg) v = pair_of(mem[g0 + m].units[0].x, mem[g0 + m].st->n_sparse);
+  for (int o = 1; o < 32; o <<= 1) {
+    const Pair u = __shfl_up_sync(0xffffffffu, v, o);
+    if (m >= o) v += u;
   }
-  if (threadIdx.x == 0) {
-    pref[M] = pair_lo(base);
-    spref[M] = pair_hi(base);
-    *work = 0;
+  if (m < Mg) {
+    pref[m + 1] = pair_lo(v);
+    spref[m + 1] = pair_hi(v);
+  }
+  if (m == 0) {
+    pref[0] = spref[0] = 0;
+    spref[Mg + 1] = 0;  // the unit counter
   }
 }
 
@@ -207,6 +210,19 @@ __global__ void __launch_bounds__(256) kb_slot_map(const BatchMember<T, U>* __re
   const long long q = (long long)(g - blk[mi]) * blockDim.x + threadIdx.x;
   if (q >= m.np) return;
   slot_one(q, m.key, m.rank, m.offset, m.perm);
+}
+
+// Scan and slot map of every member at once (resort_small_body), where each
+// has few enough keys.
+template <typename T, typename U>
+__global__ void __launch_bounds__(kSmallThreads, 2) kb_resort_small(
+    const BatchMember<T, U>* __restrict__ mem, const int* __restrict__ blk, int M) {
+  const int g = blockIdx.x;
+  const int mi = member_of(blk, M, g);
+  const BatchMember<T, U>& m = mem[mi];
+  resort_small_body(m.count, m.count_next, m.offset, m.tiles, m.units, m.nkeys, m.sparse_below,
+                    m.chunk, m.st, m.np, m.key, m.rank, m.perm, g - blk[mi],
+                    blk[mi + 1] - blk[mi]);
 }
 
 }  // namespace mithra

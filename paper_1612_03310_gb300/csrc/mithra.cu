@@ -148,8 +148,12 @@ struct mithra_sim {
 };
 
 void batch_mark_dirty(mithra_batch* b);  // defined with the batch
-// particles and column planes (32 x 8 column tiles times planes) of a batch
-void batch_totals(const mithra_batch* b, int64_t* particles, int64_t* column_planes);
+// What shares the device in a step: particles and column planes (32 x 8
+// column tiles times planes) of a simulation or a whole batch.
+struct Totals {
+  int64_t np = 0, planes = 0;
+};
+Totals batch_totals(const mithra_batch* b);
 
 namespace {
 
@@ -431,16 +435,17 @@ int unit_chunk(int64_t np, int ctas) {
 // the tiles that are split.
 int64_t unit_entries(int64_t np, int64_t nkeys) { return 1 + nkeys + np / kMinChunk; }
 
-// Particles that share the device with this simulation's: its batch's, or its
-// own.
-int64_t particles_beside(const mithra_sim* s) {
-  int64_t np = s->np, planes = 0;
-  if (s->in_batch) batch_totals(s->in_batch, &np, &planes);
-  return np;
-}
-
 int64_t column_planes(const mithra_grid& g) {
   return (int64_t)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * g.nz;
+}
+
+// The totals of the batch a simulation is in, or its own.
+Totals totals_beside(const mithra_sim* s) {
+  if (s->in_batch) return batch_totals(s->in_batch);
+  Totals t;
+  t.np = s->np;
+  t.planes = column_planes(s->g);
+  return t;
 }
 
 // Planes per CTA of the register z-marching update: the caller's, or the
@@ -451,8 +456,7 @@ int64_t column_planes(const mithra_grid& g) {
 // 40 us (2 planes); 64 x 64 x 256 cells 28 us at 16, 23 us at 8.
 int plane_run(const mithra_sim* s) {
   if (!s->lz_auto) return s->lz;
-  int64_t np = 0, planes = column_planes(s->g);
-  if (s->in_batch) batch_totals(s->in_batch, &np, &planes);
+  const int64_t planes = totals_beside(s).planes;
   const int least = s->prec == MITHRA_P64 ? 2 : 1;
   int lz = 16;
   while (lz > least && planes < (int64_t)lz * 3 * s->n_sm) lz /= 2;
@@ -472,9 +476,7 @@ int ring_run(const mithra_sim* s) {
   if (s->prec == MITHRA_P64 || !s->have_tm || s->stencil_variant != 2) return 0;
   const int cols = (s->g.nx + 31) / 32 * 32, rows = (s->g.ny + 7) / 8 * 8;
   if (10LL * s->g.nx * s->g.ny < 7LL * cols * rows) return 0;
-  int64_t np = 0, planes = column_planes(s->g);
-  if (s->in_batch) batch_totals(s->in_batch, &np, &planes);
-  if (planes < 8LL * 2 * s->n_sm) return 0;
+  if (totals_beside(s).planes < 8LL * 2 * s->n_sm) return 0;
   return s->lz_auto ? 8 : s->lz;
 }
 
@@ -489,7 +491,9 @@ int effective_run(const mithra_sim* s) {
 // the staged path's time is its number of tiles (128 x 128 x 1024 cells, 2^21
 // particles, P32_U64: 252 us at 0, 240 at 16 to 32, 273 at 64; FP64 on 96 x 80
 // x 384 cells, 4e5 particles: 536, 471 at 32, 458 at 64).  With few tiles a
-// CTA the lone warp of a sparse tile takes longer than a CTA with it.
+// CTA the lone warp of a sparse tile takes longer than a CTA with it, also in
+// a batch of many small members (64 of 32 x 32 x 128 cells and 2000
+// particles: 225 us a step staged, 238 at 32, 268 at 128).
 int sparse_below(const mithra_sim* s) {
   if (s->push_variant != 1 || !s->have_tm) return 0;
   if (s->push_sparse_below > 0) return s->push_sparse_below;
@@ -514,7 +518,7 @@ void launch_scan(mithra_sim* s, int advance, int parity, cudaStream_t q = nullpt
   int* const next = s->count[1 - parity];
   const int nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
   const int below = s->list_below = sparse_below(s);
-  const int chunk = unit_chunk(particles_beside(s), s->push_grid);
+  const int chunk = unit_chunk(totals_beside(s).np, s->push_grid);
   k_scan_partials<kRestored><<<nb, kScanBlock, 0, q>>>(cnt, s->offset, s->nkeys,
                                                        below, chunk, s->scan_part);
   k_scan_final<kRestored><<<nb, kScanBlock, 0, q>>>(cnt, next, s->offset, s->tiles, s->units,
@@ -631,7 +635,7 @@ void launch_resort(mithra_sim* s, int parity, cudaStream_t q) {
     const unsigned nb = std::min<unsigned>(blocks_for(s->np, 4 * kSmallThreads), 2 * s->n_sm);
     k_resort_small<<<nb, kSmallThreads, 0, q>>>(
         s->count[parity], s->count[1 - parity], s->offset, s->tiles, s->units, s->nkeys,
-        s->list_below, unit_chunk(particles_beside(s), s->push_grid), s->dstate, s->np, s->key,
+        s->list_below, unit_chunk(totals_beside(s).np, s->push_grid), s->dstate, s->np, s->key,
         s->rank, s->perm);
     return;
   }
@@ -1994,6 +1998,10 @@ struct mithra_batch {
   int* d_zblk = nullptr;    // boundary and update block prefixes, per group from 0
   size_t zblk_bytes = 0;
   int push_grid = 0;
+  // branches of the fused graph beside the batch's stream
+  static constexpr int kBranches = 3;
+  cudaStream_t branch[kBranches] = {nullptr, nullptr, nullptr};
+  cudaEvent_t ev_branch[kBranches] = {nullptr, nullptr, nullptr};
   // captures so far, their host time, and how many were fused
   int64_t captures = 0, fused_captures = 0;
   double capture_s = 0.0;
@@ -2003,12 +2011,13 @@ void batch_mark_dirty(mithra_batch* b) {
   if (b) b->dirty = true;
 }
 
-void batch_totals(const mithra_batch* b, int64_t* particles, int64_t* column_planes) {
-  *particles = *column_planes = 0;
+Totals batch_totals(const mithra_batch* b) {
+  Totals t;
   for (const mithra_sim* s : b->sims) {
-    *particles += s->np;
-    *column_planes += ::column_planes(s->g);
+    t.np += s->np;
+    t.planes += column_planes(s->g);
   }
+  return t;
 }
 
 namespace {
@@ -2104,7 +2113,7 @@ BatchMember<T, U> member_entry(mithra_sim* s, int c, int pb) {
   m.nkeys = s->nkeys;
   m.scan_nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
   m.sparse_below = sparse_below(s);
-  m.chunk = unit_chunk(particles_beside(s), s->push_grid);
+  m.chunk = unit_chunk(totals_beside(s).np, s->push_grid);
   m.fused_mur = s->g.boundary == 1;
   set_source_flags(s, c, &m.sp);
   m.dirty = s->dirty;
@@ -2145,6 +2154,8 @@ mithra_status capture_fused_typed(mithra_batch* b) {
   std::vector<BatchMember<T, U>> tab(2 * (size_t)M);
   std::vector<BatchMaps> maps(2 * (size_t)M);
   std::vector<int> blk((size_t)kBPCount * (M + 1), 0);
+  bool small = true;  // every member's re-sort fits the one-kernel form
+  for (const mithra_sim* s : b->sims) small = small && small_resort(s);
   for (int k = 0; k < M; ++k) {
     mithra_sim* s = b->sims[k];
     for (int t = 0; t < 2; ++t) {
@@ -2161,7 +2172,8 @@ mithra_status capture_fused_typed(mithra_batch* b) {
             ((g.nz + plane_run(s) - 1) / plane_run(s)),
         s->power_cap > 0 ? kBatchPowerBlocks : 0,
         (long long)((s->nkeys + 1 + kScanBlock - 1) / kScanBlock),
-        s->np > 0 ? (long long)blocks_for(s->np, 256) : 0};
+        small ? (long long)blocks_for(s->np, 4 * kSmallThreads)
+              : (s->np > 0 ? (long long)blocks_for(s->np, 256) : 0)};
     for (int ph = 0; ph < kBPCount; ++ph) {
       const long long v = blk[(size_t)ph * (M + 1) + k] + nb[ph];
       if (v >= (1LL << 31)) return bfail(b, MITHRA_EINVAL, "batch work list exceeds 2^31 blocks");
@@ -2228,12 +2240,21 @@ mithra_status capture_fused_typed(mithra_batch* b) {
   b->push_grid = b->sims[0]->n_sm * per_sm;
   auto total = [&](int ph) { return blk[(size_t)ph * (M + 1) + M]; };
   const int* dblk = b->d_blk;
+  for (int r = 0; r < mithra_batch::kBranches; ++r)
+    if ((!b->branch[r] &&
+         cudaStreamCreateWithFlags(&b->branch[r], cudaStreamNonBlocking) != cudaSuccess) ||
+        (!b->ev_branch[r] &&
+         cudaEventCreateWithFlags(&b->ev_branch[r], cudaEventDisableTiming) != cudaSuccess))
+      return bfail(b, MITHRA_ECUDA, "batch branch creation failed");
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return bfail(b, MITHRA_ECUDA, std::string("begin capture: ") + cudaGetErrorString(e));
   for (int t = 0; t < 2; ++t) {
     const BatchMember<T, U>* mem = static_cast<const BatchMember<T, U>*>(b->d_table) + (size_t)t * M;
     cudaStream_t q = b->stream;
+    cudaEventRecord(b->ev_branch[0], q);
+    cudaStreamWaitEvent(b->branch[0], b->ev_branch[0], 0);
+    kb_tile_prefix<T, U><<<npg, 32, 0, b->branch[0]>>>(mem, M, b->d_pref);
     // boundary and potential update, one launch each per group of up to
     // kZGroup members (their arguments in the launch's parameter space);
     // the groups' block numbers start at the group's first member
@@ -2262,34 +2283,61 @@ mithra_status capture_fused_typed(mithra_batch* b) {
         }
       }
     }
+    // the units' numbers, beside the update; then the power sample, the
+    // sparse tiles and the particle step of each group of up to kPushGroup
+    // members (their arguments in the launch's parameter space) beside each
+    // other: one group alone leaves the device partly idle (64 members of 32 x
+    // 32 x 128 cells, 2000 particles: three groups one after another 86 us)
+    auto fork = [&](int r) {
+      cudaEventRecord(b->ev_branch[r], q);
+      cudaStreamWaitEvent(b->branch[r], b->ev_branch[r], 0);
+    };
+    auto join = [&](int r) {
+      cudaEventRecord(b->ev_branch[r], b->branch[r]);
+      cudaStreamWaitEvent(q, b->ev_branch[r], 0);
+    };
+    join(0);  // the prefixes
+    bool forked[mithra_batch::kBranches] = {false, false, false};
+    auto side = [&](int r) {
+      if (!forked[r]) fork(r);
+      forked[r] = true;
+      return b->branch[r];
+    };
+    for (int r = 1; r < std::min(npg, mithra_batch::kBranches); ++r) side(r);
     if (total(kBPPow) > 0)
-      kb_power<T, U><<<total(kBPPow), 256, 0, q>>>(mem, dblk + kBPPow * (M + 1), M);
-    // the particle step, one launch per group of up to kPushGroup members
-    // (their arguments in the launch's parameter space)
-    for (int g0 = 0; g0 < M; g0 += kPushGroup) {
-      const int Mg = std::min(kPushGroup, M - g0);
-      // Mg + 1 entries of each prefix, then the counter
-      int* pref = b->d_pref + 2 * g0 + 3 * (g0 / kPushGroup);
-      int* spref = pref + Mg + 1;
-      int* work = spref + Mg + 1;
-      kb_tile_prefix<T, U><<<1, 1024, 0, q>>>(mem + g0, Mg, pref, spref, work);
-      PushParams<T, U, true> prm;
+      kb_power<T, U><<<total(kBPPow), 256, 0, side(0)>>>(mem, dblk + kBPPow * (M + 1), M);
+    std::vector<PushParams<T, U, true>> prms(npg);
+    for (int gr = 0; gr < npg; ++gr) {
+      const int g0 = gr * kPushGroup, Mg = std::min(kPushGroup, M - g0);
+      PushParams<T, U, true>& prm = prms[gr];
       for (int k = 0; k < Mg; ++k) {
         prm.m[k] = push_args_of(tab[(size_t)t * M + g0 + k]);
         prm.box[k] = maps[(size_t)t * M + g0 + k].box;
         prm.box_d[k] = maps[(size_t)t * M + g0 + k].box_d;
       }
-      prm.pref = pref;
-      prm.spref = spref;
-      prm.work = work;
+      prm.pref = prefs_of(b->d_pref, gr);
+      prm.spref = prm.pref + Mg + 1;
+      prm.work = const_cast<int*>(prm.spref) + Mg + 1;
       prm.M = Mg;
-      if (sparse) ksparse<<<sparse_grid(b->sims[0]->n_sm), kSparseThreads, 0, q>>>(prm);
-      kpush<<<b->push_grid, kPushThreads, smem, q>>>(prm);
+      if (sparse)
+        ksparse<<<sparse_grid(b->sims[0]->n_sm), kSparseThreads, 0, side(0)>>>(prm);
     }
-    kb_scan_partials<T, U><<<total(kBPScan), kScanBlock, 0, q>>>(mem, dblk + kBPScan * (M + 1), M);
-    kb_scan_final<T, U><<<total(kBPScan), kScanBlock, 0, q>>>(mem, dblk + kBPScan * (M + 1), M);
-    if (total(kBPSlot) > 0)
-      kb_slot_map<T, U><<<total(kBPSlot), 256, 0, q>>>(mem, dblk + kBPSlot * (M + 1), M);
+    for (int gr = 0; gr < npg; ++gr) {
+      const int r = gr % mithra_batch::kBranches;
+      kpush<<<b->push_grid, kPushThreads, smem, r == 0 ? q : side(r)>>>(prms[gr]);
+    }
+    for (int r = 0; r < mithra_batch::kBranches; ++r)
+      if (forked[r]) join(r);
+    if (small) {
+      kb_resort_small<T, U><<<total(kBPSlot), kSmallThreads, 0, q>>>(mem, dblk + kBPSlot * (M + 1),
+                                                                    M);
+    } else {
+      kb_scan_partials<T, U><<<total(kBPScan), kScanBlock, 0, q>>>(mem, dblk + kBPScan * (M + 1),
+                                                                  M);
+      kb_scan_final<T, U><<<total(kBPScan), kScanBlock, 0, q>>>(mem, dblk + kBPScan * (M + 1), M);
+      if (total(kBPSlot) > 0)
+        kb_slot_map<T, U><<<total(kBPSlot), 256, 0, q>>>(mem, dblk + kBPSlot * (M + 1), M);
+    }
   }
   cudaError_t le = cudaGetLastError();
   e = cudaStreamEndCapture(b->stream, &graph);
@@ -2542,6 +2590,10 @@ mithra_status mithra_batch_destroy(mithra_batch* b) {
   if (b->d_pref) cudaFree(b->d_pref);
   if (b->d_zblk) cudaFree(b->d_zblk);
   for (cudaEvent_t e : b->joins) cudaEventDestroy(e);
+  for (cudaStream_t r : b->branch)
+    if (r) cudaStreamDestroy(r);
+  for (cudaEvent_t e : b->ev_branch)
+    if (e) cudaEventDestroy(e);
   if (b->fork) cudaEventDestroy(b->fork);
   if (b->done) cudaEventDestroy(b->done);
   if (b->own_stream) cudaStreamDestroy(b->stream);

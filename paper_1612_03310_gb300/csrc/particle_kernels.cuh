@@ -861,11 +861,12 @@ constexpr int kSmallPer = 8;  // keys a thread
 constexpr int kSmallThreads = 512;
 constexpr int kSmallKeys = kSmallPer * kSmallThreads;
 
-__global__ void __launch_bounds__(kSmallThreads, 2) k_resort_small(
+// (block bidx of the nblocks that share the simulation)
+__device__ __forceinline__ void resort_small_body(
     const int* __restrict__ count, int* __restrict__ next, int* __restrict__ offset,
     int* __restrict__ tiles, int4* __restrict__ units, int nkeys, int sparse_below, int chunk,
     StepState* __restrict__ st, long long np, const int* __restrict__ key,
-    const int* __restrict__ rank, int* __restrict__ perm) {
+    const int* __restrict__ rank, int* __restrict__ perm, int bidx, int nblocks) {
   __shared__ int s_off[kSmallKeys];
   __shared__ Pair ws[32];
   // (nkeys + 1) / 512 rounded up, 1 .. kSmallPer consecutive keys a thread
@@ -887,7 +888,7 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_resort_small(
   Pair total_cu, total_ds;
   cu = block_exclusive_scan(cu, ws, &total_cu);
   ds = block_exclusive_scan(ds, ws, &total_ds);
-  const bool lists = blockIdx.x == 0;
+  const bool lists = bidx == 0;
   for (int m = 0; m < per; ++m) {
     const int t = t0 + m;
     if (t > nkeys) break;
@@ -916,12 +917,21 @@ __global__ void __launch_bounds__(kSmallThreads, 2) k_resort_small(
     st->work_sparse = 0;
     st->n += 1;
   }
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t <= nkeys; t += gridDim.x * blockDim.x)
+  for (int t = bidx * blockDim.x + threadIdx.x; t <= nkeys; t += nblocks * blockDim.x)
     next[t] = 0;
   __syncthreads();
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < np;
-       q += (long long)gridDim.x * blockDim.x)
+  for (long long q = bidx * (long long)blockDim.x + threadIdx.x; q < np;
+       q += (long long)nblocks * blockDim.x)
     perm[(long long)s_off[key[q]] + rank[q]] = (int)q;
+}
+
+__global__ void __launch_bounds__(kSmallThreads, 2) k_resort_small(
+    const int* __restrict__ count, int* __restrict__ next, int* __restrict__ offset,
+    int* __restrict__ tiles, int4* __restrict__ units, int nkeys, int sparse_below, int chunk,
+    StepState* __restrict__ st, long long np, const int* __restrict__ key,
+    const int* __restrict__ rank, int* __restrict__ perm) {
+  resort_small_body(count, next, offset, tiles, units, nkeys, sparse_below, chunk, st, np, key,
+                    rank, perm, blockIdx.x, gridDim.x);
 }
 
 // End of a step without particles: the step counter, and no source can be
