@@ -114,9 +114,9 @@ __host__ __device__ inline long long batch_mur_count(int nx, int ny, int nz, int
 
 // Potential update: block g is the member's (bx, by, bz) column tile and
 // plane run, in the register z-marching form.
-// (kMur: the members' first-order Mur at the x faces inside the loop; the
-// members of a fused batch share the boundary order.)
-template <bool kLo, typename T, bool kMur>
+// (kMur: the members' first-order Mur inside the loop, MurFused; the members
+// of a fused batch share the boundary order.)
+template <bool kLo, typename T, int kMur>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (kLo ? 3 : 4) : (kLo ? 1 : 2))
     kb_potential(const __grid_constant__ ZParams<T> prm) {
   const int g = blockIdx.x;

@@ -379,6 +379,60 @@ __global__ void __launch_bounds__(256) k_potential_step(StencilP<T> p,
   store_level<kLo>(cur, curlo, nxt, nxtlo, c, dp);
 }
 
+// kMur of the column loops: no boundary; the x faces (below); every boundary
+// vertex, by the thread of its nearest interior vertex q (for q at the x
+// faces' edges by the face's lane), which has D_q^- and D_q^+ at hand.  The
+// last saves a launch where launches and latency are what a step of a small
+// grid waits for, and k_mur_boundary's second evaluation of D_q^+ (in FP64 a
+// twentieth of the pipe's work); the ring form, whose registers are full,
+// keeps the boundary kernel.
+enum MurFused { kMurNone = 0, kMurX = 1, kMurAll = 2 };
+
+// Mur update of boundary vertex b (mask: the axes along which it lies
+// outside) from the increments qp = D_q^+, qm = D_q^- of its q, the level c
+// (lo part cl) at b.
+template <bool kLo, typename T>
+__device__ __forceinline__ void mur_store(const StencilP<T>& p, long long b, int mask, V4<T> qp,
+                                          V4<T> qm, V4<T> c, V4<T> cl, V4<T>* __restrict__ nxt,
+                                          LoV4* __restrict__ nxtlo, V4<T>* __restrict__ D,
+                                          V4<T>* __restrict__ src) {
+  V4<T> d = mur_beta0(p, mask) * (qp - D[b]) + qm;
+  if (!p.space_charge) d.w = (T)0;
+  D[b] = d;
+  if (kLo) {
+    V4<T> h, l;
+    comp_add(c, cl, d, &h, &l);
+    nxt[b] = h;
+    st_lo(nxtlo, b, l);
+  } else {
+    nxt[b] = c + d;
+  }
+  src[b] = v4((T)0, (T)0, (T)0, (T)0);
+}
+
+// The y and z boundary vertices next to vertex q = (., j, k) of a column (of
+// an x face where xb), after its update.
+template <bool kLo, typename T>
+__device__ __forceinline__ void mur_around(const StencilP<T>& p, const V4<T>* __restrict__ cur,
+                                           const LoV4* __restrict__ curlo, long long q, int j,
+                                           int k, bool xb, V4<T> qp, V4<T> qm,
+                                           V4<T>* __restrict__ nxt, LoV4* __restrict__ nxtlo,
+                                           V4<T>* __restrict__ D, V4<T>* __restrict__ src) {
+  const int yo = j == 1 ? -p.nx : (j == p.ny - 2 ? p.nx : 0);
+  const long long zo = k == 1 ? -p.nxy : (k == p.nz - 2 ? p.nxy : 0);
+  const int xm = xb ? 1 : 0;
+  auto at = [&](long long b, int mask) {
+    V4<T> cl = v4((T)0, (T)0, (T)0, (T)0);
+    if (kLo) cl = ld_lo<T>(curlo, b);
+    mur_store<kLo>(p, b, mask, qp, qm, ldg4(cur + b), cl, nxt, nxtlo, D, src);
+  };
+  if (yo != 0) at(q + yo, 2 | xm);
+  if (zo != 0) {
+    at(q + zo, 4 | xm);
+    if (yo != 0) at(q + zo + yo, 6 | xm);
+  }
+}
+
 // The FP64 column loop: bound by the FP64 pipe (2 lanes a clock and SM), so
 // the same update in fewer operations.  A plane brings one combination
 // t = rxA X + ryA Y (a = t, b = kap t, kap = (1 - 2A)/A: both weights of the
@@ -386,7 +440,7 @@ __global__ void __launch_bounds__(256) k_potential_step(StencilP<T> p,
 // the z difference of a plane serves the next one, and a tile without
 // sources skips their terms: 15 operations a vertex and component instead
 // of 19.  96 x 80 x 384 cells: potential scope 577 -> 482 us.
-template <bool kMur>
+template <int kMur>
 __device__ __forceinline__ void zloop_body64(const StencilP<double>& p,
                                              const V4<double>* __restrict__ cur,
                                              V4<double>* __restrict__ nxt,
@@ -445,17 +499,20 @@ __device__ __forceinline__ void zloop_body64(const StencilP<double>& p,
         L = vfma4<false>(v4(p.sA, p.sA, p.sA, p.sphi), sv, L);
       }
     }
-    D4 dp = dm + L;
+    D4 dp = dm + L, qp = dp, qm = dm;
     if (kMur && xwarp) {  // warp-uniform
-      const D4 dq = v4(__shfl_sync(live, dp.x, from), __shfl_sync(live, dp.y, from),
-                       __shfl_sync(live, dp.z, from), __shfl_sync(live, dp.w, from));
-      const D4 mq = v4(__shfl_sync(live, dm.x, from), __shfl_sync(live, dm.y, from),
-                       __shfl_sync(live, dm.z, from), __shfl_sync(live, dm.w, from));
-      if (xb) dp = mur_beta0(p, 1) * (dq - dm) + mq;
+      qp = v4(__shfl_sync(live, dp.x, from), __shfl_sync(live, dp.y, from),
+              __shfl_sync(live, dp.z, from), __shfl_sync(live, dp.w, from));
+      qm = v4(__shfl_sync(live, dm.x, from), __shfl_sync(live, dm.y, from),
+              __shfl_sync(live, dm.z, from), __shfl_sync(live, dm.w, from));
+      if (xb) dp = mur_beta0(p, 1) * (qp - dm) + qm;
     }
     if (!p.space_charge) dp.w = 0.0;
     D[q] = dp;
     nxt[q] = c0 + dp;
+    if (kMur == kMurAll)
+      mur_around<false>(p, cur, (const LoV4*)nullptr, q, j, k, xb, qp, qm, nxt, (LoV4*)nullptr,
+                        D, src);
     ab = nsfd ? vfma<false>(p.kap, tp, a0) : tp;
     a0 = nsfd ? tp : zero;
     dz0 = dz;
@@ -470,7 +527,7 @@ __device__ __forceinline__ void zloop_body64(const StencilP<double>& p,
 // by warp shuffle: D_b^+ = b0 (D_q^+ - D_b^-) + D_q^-.  Their loads fall in
 // the rows the warp reads anyway; every other boundary vertex is left to
 // k_mur_boundary<.., kRest = true>.
-template <bool kLo, typename T, bool kMur>
+template <bool kLo, typename T, int kMur>
 __device__ __forceinline__ void zloop_body(const StencilP<T>& p, const V4<T>* __restrict__ cur,
                                            const LoV4* __restrict__ curlo,
                                            V4<T>* __restrict__ nxt, LoV4* __restrict__ nxtlo,
@@ -537,12 +594,13 @@ __device__ __forceinline__ void zloop_body(const StencilP<T>& p, const V4<T>* __
     V4<T> sv = v4((T)0, (T)0, (T)0, (T)0);
     if (src_every || p.dirty[(k >> 3) * ntxy + trow] != 0) sv = src[q];
     V4<T> dp = next_increment<!kLo>(p, dm, L, sv);
+    V4<T> qp = dp, qm = dm;
     if (kMur && xwarp) {  // warp-uniform
-      const V4<T> dq = v4(__shfl_sync(live, dp.x, from), __shfl_sync(live, dp.y, from),
-                          __shfl_sync(live, dp.z, from), __shfl_sync(live, dp.w, from));
-      const V4<T> mq = v4(__shfl_sync(live, dm.x, from), __shfl_sync(live, dm.y, from),
-                          __shfl_sync(live, dm.z, from), __shfl_sync(live, dm.w, from));
-      if (xb) dp = mur_beta0(p, 1) * (dq - dm) + mq;
+      qp = v4(__shfl_sync(live, dp.x, from), __shfl_sync(live, dp.y, from),
+              __shfl_sync(live, dp.z, from), __shfl_sync(live, dp.w, from));
+      qm = v4(__shfl_sync(live, dm.x, from), __shfl_sync(live, dm.y, from),
+              __shfl_sync(live, dm.z, from), __shfl_sync(live, dm.w, from));
+      if (xb) dp = mur_beta0(p, 1) * (qp - dm) + qm;
     }
     if (!p.space_charge) dp.w = (T)0;
     if (nonzero(sv)) src[q] = v4((T)0, (T)0, (T)0, (T)0);
@@ -555,6 +613,8 @@ __device__ __forceinline__ void zloop_body(const StencilP<T>& p, const V4<T>* __
     } else {
       nxt[q] = vadd<true>(c0, dp);
     }
+    if (kMur == kMurAll)
+      mur_around<kLo>(p, cur, curlo, q, j, k, xb, qp, qm, nxt, nxtlo, D, src);
     ab = vadd<!kLo>(a0, tp.b);
     a0 = tp.a;
     cm = c0; clm = cl0; c0 = tp.c; cl0 = tp.cl;
@@ -569,19 +629,21 @@ __global__ void __launch_bounds__(256) k_potential_zloop(StencilP<T> p,
                                                          LoV4* __restrict__ nxtlo,
                                                          V4<T>* __restrict__ D,
                                                          V4<T>* __restrict__ src, int lz) {
-  zloop_body<kLo, T, false>(p, cur, curlo, nxt, nxtlo, D, src, lz, blockIdx.x, blockIdx.y,
+  zloop_body<kLo, T, kMurNone>(p, cur, curlo, nxt, nxtlo, D, src, lz, blockIdx.x, blockIdx.y,
                             blockIdx.z);
 }
 
-// The same with first-order Mur fused; the register caps keep the
-// occupancy of the plain form.
-template <bool kLo, typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (kLo ? 3 : 4) : (kLo ? 1 : 2))
+// The same with first-order Mur fused (kMurX or kMurAll); the register caps
+// of the x faces' form keep the occupancy of the plain form.
+template <bool kLo, typename T, int kMur>
+__global__ void __launch_bounds__(256, kMur == kMurAll ? (sizeof(T) == 4 ? 2 : 1)
+                                       : sizeof(T) == 4 ? (kLo ? 3 : 4)
+                                                        : (kLo ? 1 : 2))
     k_potential_zloop_mur1(StencilP<T> p, const V4<T>* __restrict__ cur,
                            const LoV4* __restrict__ curlo, V4<T>* __restrict__ nxt,
                            LoV4* __restrict__ nxtlo, V4<T>* __restrict__ D,
                            V4<T>* __restrict__ src, int lz) {
-  zloop_body<kLo, T, true>(p, cur, curlo, nxt, nxtlo, D, src, lz, blockIdx.x, blockIdx.y,
+  zloop_body<kLo, T, kMur>(p, cur, curlo, nxt, nxtlo, D, src, lz, blockIdx.x, blockIdx.y,
                            blockIdx.z);
 }
 

@@ -480,6 +480,15 @@ int ring_run(const mithra_sim* s) {
   return s->lz_auto ? 8 : s->lz;
 }
 
+// Whether the register z-marching update of a simulation of its own does
+// every boundary vertex itself (kMurAll): always where that form is used, as
+// it is in FP32 on small grids and in FP64 (potential scope with the boundary
+// kernel and without: 32 x 32 x 64 cells 11.5 and 8.1 us, in FP64 37 and 23;
+// 96 x 80 x 384 in FP64 483 and 451), unless the x+ face's lanes cannot share
+// a warp with their neighbours.  A fused batch keeps the boundary kernel (64
+// members of 32 x 32 x 128 cells: 212 us a step with it, 217 without).
+bool mur_all(const mithra_sim* s) { return s->g.boundary == 1 && xhi_fused(s->g.nx); }
+
 // Planes per CTA that the single simulation's z-marching update takes.
 int effective_run(const mithra_sim* s) {
   const int ring = ring_run(s);
@@ -682,9 +691,13 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
     // beside the z-marching form the boundary recomputes D_q^+ in its
     // arithmetic
     const bool zm = s->stencil_variant == 2;
+    const int rl = ring_run(s);
+    const bool all = fused && rl == 0 && mur_all(s);
     const dim3 mg = mur_grid(s->g.nx, s->g.ny, s->g.nz);
     const unsigned rg = blocks_for(rest_count(s->g.nx, s->g.ny, s->g.nz), 256);
-    if (fused && L0)
+    if (all) {
+      // every boundary vertex by the update itself
+    } else if (fused && L0)
       k_mur_boundary<true, T, true, true><<<rg, 256, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S);
     else if (fused)
       k_mur_boundary<false, T, true, true><<<rg, 256, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S);
@@ -702,7 +715,6 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
       const int lz = plane_run(s);
       dim3 blk(32, 8, 1);
       dim3 grd((s->g.nx + 31) / 32, (s->g.ny + 7) / 8, (s->g.nz + lz - 1) / lz);
-      const int rl = ring_run(s);
       if constexpr (sizeof(T) == 4) {
         if (rl > 0) {
           const int lo = !L0 ? kRingPlain : (s->have_lo_map ? kRingTma : kRingAsync);
@@ -721,12 +733,18 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
       }
       if (rl > 0) {
         // launched above
-      } else if (L0 && fused)
-        k_potential_zloop_mur1<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
+      } else if (L0 && all)
+        k_potential_zloop_mur1<true, T, kMurAll><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1,
+                                                                            Dn, S, lz);
+      else if (all)
+        k_potential_zloop_mur1<false, T, kMurAll><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1,
+                                                                             Dn, S, lz);
+      else if (L0 && fused)
+        k_potential_zloop_mur1<true, T, kMurX><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else if (L0)
         k_potential_zloop<true, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else if (fused)
-        k_potential_zloop_mur1<false, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
+        k_potential_zloop_mur1<false, T, kMurX><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
       else
         k_potential_zloop<false, T><<<grd, blk, 0, s->stream>>>(sp, P0, L0, P1, L1, Dn, S, lz);
     } else if (s->stencil_variant == 1 && s->have_tm && !L0) {
@@ -2274,12 +2292,12 @@ mithra_status capture_fused_typed(mithra_batch* b) {
         if (ph == kBPMur) {
           if (lo) kb_mur<kAnyLo, T><<<nblk, 256, 0, q>>>(zp);
           else kb_mur<false, T><<<nblk, 256, 0, q>>>(zp);
-        } else if (b->sims[0]->g.boundary == 1) {
-          if (lo) kb_potential<kAnyLo, T, true><<<nblk, dim3(32, 8), 0, q>>>(zp);
-          else kb_potential<false, T, true><<<nblk, dim3(32, 8), 0, q>>>(zp);
         } else {
-          if (lo) kb_potential<kAnyLo, T, false><<<nblk, dim3(32, 8), 0, q>>>(zp);
-          else kb_potential<false, T, false><<<nblk, dim3(32, 8), 0, q>>>(zp);
+          auto kz = b->sims[0]->g.boundary == 1
+                        ? (lo ? kb_potential<kAnyLo, T, kMurX> : kb_potential<false, T, kMurX>)
+                        : (lo ? kb_potential<kAnyLo, T, kMurNone>
+                              : kb_potential<false, T, kMurNone>);
+          kz<<<nblk, dim3(32, 8), 0, q>>>(zp);
         }
       }
     }

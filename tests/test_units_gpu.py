@@ -163,3 +163,28 @@ def test_sparse_threshold_switched_off(M, orc, fused):  # noqa: F811
             sim.sync()
             compare_fields(sim, o, 1e-5, names=["Ex", "Bz", "phi", "Jx", "rho"])
             compare_particles(sim, o, 2e-5, 1e-5)
+
+
+@pytest.mark.parametrize("prec", ["P64", "P32", "P32_C"])
+@pytest.mark.parametrize("shape", [(4, 4, 4), (5, 4, 7), (33, 6, 9), (32, 8, 4), (34, 9, 16),
+                                   (64, 5, 6), (65, 17, 12)])
+def test_update_with_its_boundary(M, orc, prec, shape):  # noqa: F811
+    # small grids, where the register form updates every boundary vertex
+    # itself (nx - 1 a multiple of 32: the boundary kernel's part): corners
+    # and edges of grids down to two interior vertices an axis, every vertex
+    # compared
+    g = dict(inputs.random_grid(95, *shape), boundary=1)
+    f = inputs.random_fields(96, g, scale=1e-9)
+    if prec != "P64":
+        f = {k: v.astype(np.float32).astype(np.float64) for k, v in f.items()}
+    o = orc.OracleSim(g, None, dict(x=[], y=[], z=[], ux=[], uy=[], uz=[]))
+    with M.Simulation(g, None, None, precision=getattr(M, prec)) as sim:
+        set_state(sim, o, f)
+        for n in (1, 2):
+            o.step(n)
+            sim.step(n)
+            sim.sync()
+            for nm in ("Ax", "Ay", "Az", "phi", "Ax_prev"):
+                ref = oracle_fields(o)[nm]
+                tol = 1e-12 if prec == "P64" else 1e-5
+                assert np.abs(sim.copy_field(nm) - ref).max() <= tol * np.abs(ref).max(), nm
