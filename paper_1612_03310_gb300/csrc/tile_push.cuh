@@ -307,7 +307,10 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   int* sl_pos = sl_id + kPushThreads;
   int* sRh = reinterpret_cast<int*>(sP);
   int* sRl = sRh + kTPC;
-  __shared__ int s_tile;
+  // this CTA's units {tile (-1: none left), first slot, end slot, member}:
+  // the one in work and the next
+  __shared__ int4 s_unit[2];
+  __shared__ int s_claim;
   __shared__ UndFrame<T> s_frame[kMaxFrames];  // undulator frames of the tile
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -358,9 +361,37 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   // the units of one simulation's list, then its sparse tiles and lost
   // tail (each written once; one simulation runs them straight through, a
   // batch member by member)
-  // one staged unit: entry t of the simulation's unit list
+  // units of the launch
+  auto units = [&]() {
+    if constexpr (kBatch) return prm.pref[prm.M];
+    else return prm.args.units[0].x;
+  };
+  // unit number w of the launch
+  auto unit_of = [&](int w) {
+    if (w >= units()) return make_int4(-1, 0, 0, 0);
+    if constexpr (!kBatch) {
+      return prm.args.units[1 + w];
+    } else {
+      const int mi = member_of_tile(prm.pref, prm.M, w);
+      const int4 u = prm.m[mi].units[1 + w - prm.pref[mi]];
+      return make_int4(u.x, u.y, u.z, mi);
+    }
+  };
+  auto counter = [&]() {
+    if constexpr (kBatch) return prm.work;
+    else return &prm.args.st->work;
+  };
+  // one staged unit.  Its last warp's first lane takes the CTA's next unit
+  // meanwhile, so that the two round trips to L2 (the counter's atomic, the
+  // list's entry) do not stand between two units: under the charge block's
+  // flush, or, for units of one round of particles in a list of many per CTA,
+  // under the boxes' flight and the E/B phase (taken that early, the last
+  // units wait for CTAs still at work: c2, 7 units a CTA, 240 -> 248 us; 64
+  // batch members of 2000 particles, 14 a CTA, 225 -> 210 us a step).
+  constexpr int kClaim = kPushThreads - 32;
+  const bool many = units() >= 10 * (int)gridDim.x;
   auto dense = [&](const PushArgs<T, U>& a, const CUtensorMap* tmp, const CUtensorMap* tmd,
-                   int t, double th) {
+                   const int4 unit, double th) {
     const PicP<T>& p = a.p;
     StepState* const& st = a.st;
     const V4<T>* const& pn = a.pn;
@@ -374,7 +405,6 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
     int* const& rank = a.rank;
     long long* const& lost_ctr = a.lost_ctr;
     {
-      const int4 unit = a.units[1 + t];
       const int tile = unit.x, beg = unit.y, end = unit.z;
       int i0, j0, k0;
       tile_origin(p, tile, &i0, &j0, &k0);
@@ -384,6 +414,8 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
         tma_load_field(sP, tmp, i0 - 1, j0 - 1, k0 - 1, bar);
         tma_load_field(sD, tmd, i0 - 1, j0 - 1, k0 - 1, bar);
       }
+      const bool early = many && end - beg <= kPushThreads;
+      if (early && tid == kClaim) s_claim = (int)gridDim.x + atomicAdd(counter(), 1);
       if (tid < 27) mark_tile(a, tile, tid);
       // the lo parts of psi^{n+1}, which the E/B phase reads from global
       // memory (the update that wrote them has since streamed the grid
@@ -402,6 +434,7 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
         s_frame[m] = und_frame(p, k0, th + m * p.dtb);
       mbar_wait_bounded(bar, phase, &st->err);
       phase ^= 1u;
+      if (early && tid == kClaim) s_unit[phase] = unit_of(s_claim);
       // E and B at the tile's vertices
       for (int v = tid; v < kTEC; v += blockDim.x) {
         const int a = v % kTE, b = (v / kTE) % kTE, c = v / (kTE * kTE);
@@ -477,6 +510,8 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
             });
       }
       __syncthreads();
+      if (!early && tid == kClaim)
+        s_unit[phase] = unit_of((int)gridDim.x + atomicAdd(counter(), 1));
       // add the block to the global sources (touched vertices only)
       if (kF32) {
         const float s1 = (float)p.qV * __int_as_float((127 - bsh) << 23);
@@ -493,24 +528,23 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
       __syncthreads();
     }
   };
+  // the CTA's first unit by its number, the others from the counter
+  if (tid == 0) s_unit[0] = unit_of(blockIdx.x);
   if constexpr (!kBatch) {
     const PushArgs<T, U>& a = prm.args;
     clear_flags(a, blockIdx.x, gridDim.x);
-    const int nunits = a.units[0].x;
+    __syncthreads();
     const double th = a.p.t0 + ((double)a.st->n + 0.5) * a.p.dt;
-    for (;;) {  // the CTA takes units from the list until none is left
-      if (tid == 0) s_tile = atomicAdd(&a.st->work, 1);
-      __syncthreads();
-      const int t = s_tile;
-      if (t >= nunits) break;
-      dense(a, &prm.tm_pn, &prm.tm_d, t, th);
+    for (;;) {
+      const int4 unit = s_unit[phase];
+      if (unit.x < 0) break;
+      dense(a, &prm.tm_pn, &prm.tm_d, unit, th);
     }
     // particles lost before this step sit at the tail of the sorted order (the
     // bucket after the last tile); they keep that bucket in the re-sort
     lost_tail(a, blockIdx.x, gridDim.x);
   } else {
-    // the group's units from one counter; the CTAs share the members for the
-    // flags and the lost tails
+    // the CTAs share the members for the flags and the lost tails
     const int M = prm.M;
     const int share = max((int)gridDim.x / M, 1);
     auto each_member = [&](auto&& f) {
@@ -522,15 +556,13 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
       }
     };
     each_member(clear_flags);
+    __syncthreads();
     for (;;) {
-      if (tid == 0) s_tile = atomicAdd(prm.work, 1);
-      __syncthreads();
-      const int w = s_tile;
-      if (w >= prm.pref[M]) break;
-      const int mi = member_of_tile(prm.pref, M, w);
-      const PushArgs<T, U>& a = prm.m[mi];
+      const int4 unit = s_unit[phase];
+      if (unit.x < 0) break;
+      const PushArgs<T, U>& a = prm.m[unit.w];
       const double th = a.p.t0 + ((double)a.st->n + 0.5) * a.p.dt;
-      dense(a, &prm.box[mi], &prm.box_d[mi], w - prm.pref[mi], th);
+      dense(a, &prm.box[unit.w], &prm.box_d[unit.w], unit, th);
     }
     // the particles each member lost before this step keep their bucket
     each_member(lost_tail);
