@@ -304,8 +304,7 @@ const char* mithra_kernel_name(int32_t kernel);
  * sources of every other tile are zero.  *marked receives the number of
  * tiles marked for the next step, *everywhere 1 when that update reads the
  * sources of every vertex instead (after the initial deposit, a step of the
- * per-particle form, a set or restored source field, or a deposit further
- * than one tile from its particle's tile) and 0 otherwise.  Waits for the
+ * per-particle form, or a set or restored source field) and 0 otherwise.  Waits for the
  * simulation's stream.  Errors: MITHRA_EINVAL for a NULL argument,
  * MITHRA_ECUDA when a copy fails. */
 mithra_status mithra_source_tiles(mithra_sim* sim, int64_t* marked, int32_t* everywhere);

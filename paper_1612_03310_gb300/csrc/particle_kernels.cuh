@@ -16,7 +16,21 @@ __device__ inline void sincos_t(double a, double* s, double* c) { sincos(a, s, c
 // cosh and sinh of the same argument from one expm1: with m = e^a - 1,
 // sinh a = m (1 + e^{-a}) / 2 (no cancellation for small a) and
 // cosh a = (e^a + e^{-a}) / 2.
+// For |a| <= 1/2 (ku y of a beam near the axis) the Taylor series, whose next
+// terms are 0.5^10/10! = 3e-10 and 0.5^9/9! / 0.5 = 1e-8.
 __device__ inline void coshsinh_t(float a, float* ch, float* sh) {
+  if (fabsf(a) <= 0.5f) {
+    const float q = a * a;
+    float c = fmaf(1.0f / 40320.0f, q, 1.0f / 720.0f);
+    float s = fmaf(1.0f / 362880.0f, q, 1.0f / 5040.0f);
+    c = fmaf(c, q, 1.0f / 24.0f);
+    s = fmaf(s, q, 1.0f / 120.0f);
+    c = fmaf(c, q, 0.5f);
+    s = fmaf(s, q, 1.0f / 6.0f);
+    *ch = fmaf(c, q, 1.0f);
+    *sh = fmaf(s * q, a, a);
+    return;
+  }
   const float m = expm1f(a);
   const float inv = 1.0f / (1.0f + m);
   *ch = 0.5f * ((1.0f + m) + inv);
@@ -221,6 +235,36 @@ __device__ inline FF ff_mul(FF a, float b) {
   return ff_fast(p.hi, p.lo + a.lo * b);
 }
 
+// 1 + a.a of a float-float vector, and a component b d - c e of a float-float
+// cross product: the leading products split exactly, summed by TwoSum, every
+// remainder and cross term in the low word, one renormalization at the end
+// (fewer operations than sums of renormalized pairs, to the same ~2^-46 of
+// the largest term).
+__device__ inline FF ff_one_plus_dot(const FF a[3]) {
+  float hi = 1.0f, lo = 0.0f;
+#pragma unroll
+  for (int m = 0; m < 3; ++m) {
+    const FF p = ff_prod(a[m].hi, a[m].hi);
+    const FF s = ff_two_sum(hi, p.hi);
+    lo += s.lo + fmaf(2.0f * a[m].hi, a[m].lo, p.lo);
+    hi = s.hi;
+  }
+  return ff_fast(hi, lo);
+}
+__device__ inline FF ff_cross(FF b, FF d, FF c, FF e) {
+  const FF p = ff_prod(b.hi, d.hi), q = ff_prod(c.hi, e.hi);
+  const FF s = ff_two_sum(p.hi, -q.hi);
+  const float x = fmaf(b.hi, d.lo, fmaf(b.lo, d.hi, p.lo));
+  const float y = fmaf(c.hi, e.lo, fmaf(c.lo, e.hi, q.lo));
+  return ff_fast(s.hi, s.lo + (x - y));
+}
+// a + b + c
+__device__ inline FF ff_add3(FF a, FF b, FF c) {
+  const FF s = ff_two_sum(a.hi, b.hi);
+  const FF t = ff_two_sum(s.hi, c.hi);
+  return ff_fast(t.hi, (s.lo + t.lo) + ((a.lo + b.lo) + c.lo));
+}
+
 // 1/sqrt(x) for x >= 1 in FP64 by the Newton-Raphson iteration for the
 // reciprocal square root, y <- y (3 - x y^2) / 2, from an FP32 seed (rsqrtf):
 // the error squares each step, one step reaches ~1e-13, two reach FP64
@@ -354,27 +398,24 @@ __device__ inline void boris_ff(const PicP<float>& p, FF u[3], const float Ef[3]
   const FF hE[3] = {ff_mul(h, Ef[0]), ff_mul(h, Ef[1]), ff_mul(h, Ef[2])};
   const FF t1[3] = {ff_add(u[0], hE[0]), ff_add(u[1], hE[1]), ff_add(u[2], hE[2])};
   // 1 / gamma_1 = 1 / sqrt(1 + t1.t1)
-  const FF g2 = ff_add(ff_add(ff_add(FF{1.0f, 0.0f}, ff_mul(t1[0], t1[0])), ff_mul(t1[1], t1[1])),
-                       ff_mul(t1[2], t1[2]));
+  const FF g2 = ff_one_plus_dot(t1);
   const float y0 = rsqrtf(g2.hi);
   const FF e1 = ff_sub(FF{1.0f, 0.0f}, ff_mul(g2, ff_prod(y0, y0)));  // 1 - g2 y0^2, small
   const FF ig1 = ff_two_sum(y0, 0.5f * y0 * e1.hi);
   const FF al = ff_mul(an, ig1);
   const FF t[3] = {ff_mul(al, Bf[0]), ff_mul(al, Bf[1]), ff_mul(al, Bf[2])};
   // f = 2 / (1 + t.t)
-  const FF den = ff_add(ff_add(ff_add(FF{1.0f, 0.0f}, ff_mul(t[0], t[0])), ff_mul(t[1], t[1])),
-                        ff_mul(t[2], t[2]));
+  const FF den = ff_one_plus_dot(t);
   const float r0 = 1.0f / den.hi;
   const FF e2 = ff_sub(FF{1.0f, 0.0f}, ff_mul(den, r0));  // 1 - den r0, small
   const FF f = ff_two_sum(2.0f * r0, 2.0f * r0 * e2.hi);
   const FF sv[3] = {ff_mul(f, t[0]), ff_mul(f, t[1]), ff_mul(f, t[2])};
-  const FF t2[3] = {ff_add(t1[0], ff_sub(ff_mul(t1[1], t[2]), ff_mul(t1[2], t[1]))),
-                    ff_add(t1[1], ff_sub(ff_mul(t1[2], t[0]), ff_mul(t1[0], t[2]))),
-                    ff_add(t1[2], ff_sub(ff_mul(t1[0], t[1]), ff_mul(t1[1], t[0])))};
-  const FF c[3] = {ff_sub(ff_mul(t2[1], sv[2]), ff_mul(t2[2], sv[1])),
-                   ff_sub(ff_mul(t2[2], sv[0]), ff_mul(t2[0], sv[2])),
-                   ff_sub(ff_mul(t2[0], sv[1]), ff_mul(t2[1], sv[0]))};
-  for (int a = 0; a < 3; ++a) u[a] = ff_add(ff_add(t1[a], c[a]), hE[a]);
+  const FF t2[3] = {ff_add(t1[0], ff_cross(t1[1], t[2], t1[2], t[1])),
+                    ff_add(t1[1], ff_cross(t1[2], t[0], t1[0], t[2])),
+                    ff_add(t1[2], ff_cross(t1[0], t[1], t1[1], t[0]))};
+  const FF c[3] = {ff_cross(t2[1], sv[2], t2[2], sv[1]), ff_cross(t2[2], sv[0], t2[0], sv[2]),
+                   ff_cross(t2[0], sv[1], t2[1], sv[0])};
+  for (int a = 0; a < 3; ++a) u[a] = ff_add3(t1[a], c[a], hE[a]);
 }
 
 template <>

@@ -146,11 +146,11 @@ __device__ inline void deposit_rho_fixed(const PicP<T>& p, int* __restrict__ hi,
 // through dep(kRho, i, j, k, f, jx, jy, jz, rho), and the re-sort bucket.
 // The particle in slot q of the tile order comes from ld_cell(), ld_fu(f, u)
 // and ld_id() (the state buffer at the slot's position) and goes to slot q
-// of the output buffer O, complete (a lost particle too), so that O holds
-// every particle in slot order.  next() is called once the state has been
-// consumed (after the push, or for a lost particle after its loads), where
-// the dense loop starts the copy of the thread's next particle into the
-// slot it read.
+// of the output buffer O, complete (one that is lost in this step too), so
+// that O holds every particle in slot order.  A tile's slots hold no particle
+// lost before (those have a bucket of their own, lost_tail).  next() is called
+// once the state has been consumed, where the dense loop starts the copy of
+// the thread's next particle into the slot it read.
 template <bool kOpt, typename T, typename U, typename Gather, typename Frame, typename Dep,
           typename LdCell, typename LdFU, typename LdId, typename Next>
 __device__ inline void tile_particle(const PicP<T>& p, const Parts<T, U>& O, long long q,
@@ -158,51 +158,39 @@ __device__ inline void tile_particle(const PicP<T>& p, const Parts<T, U>& O, lon
                                      int* __restrict__ rank, long long* __restrict__ lost_ctr,
                                      Gather&& gather, Frame&& frame, Dep&& dep, LdCell&& ld_cell,
                                      LdFU&& ld_fu, LdId&& ld_id, Next&& next) {
-  const int cell = ld_cell();
-  const int id = ld_id();
+  int i, j, k;
+  decode_cell(p, ld_cell(), &i, &j, &k);
+  O.id[q] = ld_id();
   T f[3];
   U u[3];
   ld_fu(f, u);
-  O.id[q] = id;
-  int kk = p.nkeys;
-  if (cell < 0) {
-    next();
-    O.cell[q] = cell;
-    O.fx[q] = f[0]; O.fy[q] = f[1]; O.fz[q] = f[2];
-    O.ux[q] = u[0]; O.uy[q] = u[1]; O.uz[q] = u[2];
-  } else {
-    int i, j, k;
-    decode_cell(p, cell, &i, &j, &k);
-    const int ia = i, ja = j, ka = k;
-    const T f0[3] = {f[0], f[1], f[2]};
-    T disp[3];
-    const bool ok = push_particle<kOpt>(p, i, j, k, f, u, disp, gather, frame);
-    next();
-    O.ux[q] = u[0]; O.uy[q] = u[1]; O.uz[q] = u[2];
-    if (!ok) {
-      O.cell[q] = -1;
-      O.fx[q] = f0[0]; O.fy[q] = f0[1]; O.fz[q] = f0[2];
-      atomicAdd(reinterpret_cast<unsigned long long*>(lost_ctr), 1ULL);
-    } else {
-      O.cell[q] = (int)cidx(i, j, k, p.nx, p.nxy);
-      O.fx[q] = f[0]; O.fy[q] = f[1]; O.fz[q] = f[2];
-      // the bucket's rank first: its atomic's round trip overlaps the
-      // deposits
-      kk = tile_key(p, i, j, k);
-      const int r = bin_rank(count, kk);
-      dep(true, i, j, k, f, (T)0, (T)0, (T)0, p.qV);
-      T mf[3];
-      const int mi = split_cell_t(ia, f0[0] + (T)0.5 * disp[0], &mf[0]);
-      const int mj = split_cell_t(ja, f0[1] + (T)0.5 * disp[1], &mf[1]);
-      const int mk = split_cell_t(ka, f0[2] + (T)0.5 * disp[2], &mf[2]);
-      dep(false, mi, mj, mk, mf, p.jx * disp[0], p.jy * disp[1], p.jz * disp[2], (T)0);
-      key[q] = kk;
-      rank[q] = r;
-      return;
-    }
+  const int ia = i, ja = j, ka = k;
+  const T f0[3] = {f[0], f[1], f[2]};
+  T disp[3];
+  const bool ok = push_particle<kOpt>(p, i, j, k, f, u, disp, gather, frame);
+  next();
+  O.ux[q] = u[0]; O.uy[q] = u[1]; O.uz[q] = u[2];
+  if (!ok) {
+    O.cell[q] = -1;
+    O.fx[q] = f0[0]; O.fy[q] = f0[1]; O.fz[q] = f0[2];
+    atomicAdd(reinterpret_cast<unsigned long long*>(lost_ctr), 1ULL);
+    key[q] = p.nkeys;
+    rank[q] = bin_rank(count, p.nkeys);
+    return;
   }
+  O.cell[q] = (int)cidx(i, j, k, p.nx, p.nxy);
+  O.fx[q] = f[0]; O.fy[q] = f[1]; O.fz[q] = f[2];
+  // the bucket's rank first: its atomic's round trip overlaps the deposits
+  const int kk = tile_key(p, i, j, k);
+  const int r = bin_rank(count, kk);
+  dep(true, i, j, k, f, (T)0, (T)0, (T)0, p.qV);
+  T mf[3];
+  const int mi = split_cell_t(ia, f0[0] + (T)0.5 * disp[0], &mf[0]);
+  const int mj = split_cell_t(ja, f0[1] + (T)0.5 * disp[1], &mf[1]);
+  const int mk = split_cell_t(ka, f0[2] + (T)0.5 * disp[2], &mf[2]);
+  dep(false, mi, mj, mk, mf, p.jx * disp[0], p.jy * disp[1], p.jz * disp[2], (T)0);
   key[q] = kk;
-  rank[q] = bin_rank(count, kk);
+  rank[q] = r;
 }
 
 template <typename T>
@@ -253,9 +241,8 @@ struct PushParams<T, U, true> {
 
 // Source-tile flags (StencilP::dirty): the deposits mark the flags of the
 // next update -- a tile's 27 neighbours, which hold every vertex a particle
-// of the tile deposits to while its end and mid-point cells stay within
-// [t0 - 8, t0 + 14] on each axis (t0 the tile's first cell); a deposit beyond
-// that sets src_all of the next parity instead.
+// of the tile deposits to: c dt is below every spacing (mithra_check_grid),
+// so that a step moves a particle by less than a cell along each axis.
 template <typename T, typename U>
 __device__ inline void mark_tile(const PushArgs<T, U>& a, int tile, int r) {  // neighbour r of 27
   const PicP<T>& p = a.p;
@@ -264,14 +251,6 @@ __device__ inline void mark_tile(const PushArgs<T, U>& a, int tile, int r) {  //
   if (tx >= 0 && tx < p.ntx && ty >= 0 && ty < p.nty && tz >= 0 && tz < p.ntz)
     a.dirty[(size_t)(1 - a.cur) * 4 * a.dirty_words + ((size_t)tz * p.nty + ty) * p.ntx + tx] = 1;
 }
-template <typename T, typename U>
-__device__ inline void far_deposit(const PushArgs<T, U>& a, int i0, int j0, int k0, int i, int j,
-                                   int k) {
-  if ((unsigned)(i - i0 + 8) > 22u || (unsigned)(j - j0 + 8) > 22u ||
-      (unsigned)(k - k0 + 8) > 22u)
-    a.st->src_all[1 - a.cur] = 1;
-}
-
 constexpr int kMaxFrames = 16;  // undulator frames kept per tile (sub-steps)
 
 template <bool kOpt, typename T, typename U, bool kLo = false, bool kBatch = false>
@@ -324,7 +303,7 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   asm volatile("griddepcontrol.wait;" ::: "memory");
   uint32_t phase = 0;
   // Source-tile flags: the array this step's potential update read is
-  // cleared, and the deposits mark the other (mark_tile, far_deposit)
+  // cleared, and the deposits mark the other (mark_tile)
   // (done by CTA b of the nb that share the simulation)
   auto clear_flags = [&](const PushArgs<T, U>& a, int b, int nb) {
     unsigned* f = reinterpret_cast<unsigned*>(a.dirty) + (size_t)a.cur * a.dirty_words;
@@ -490,7 +469,6 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
               return m < kMaxFrames ? s_frame[m] : und_frame(p, k0, th + m * p.dtb);
             },
             [&](bool rho, int i, int j, int k, const T* f, T jx, T jy, T jz, T q) {
-              far_deposit(a, i0, j0, k0, i, j, k);
               if (!rho)
                 deposit_j(p, src, i, j, k, f[0], f[1], f[2], jx, jy, jz);
               else if constexpr (kF32)
@@ -601,7 +579,6 @@ __device__ inline void push_sparse_tile(const PushArgs<T, U>& a, int tile, doubl
           return m < kMaxFrames ? wf[m] : und_frame(p, k0, th + m * p.dtb);
         },
         [&](bool rho, int i, int j, int k, const T* f, T jx, T jy, T jz, T q) {
-          far_deposit(a, i0, j0, k0, i, j, k);
           if (rho)
             deposit_rho(p, src, i, j, k, f[0], f[1], f[2], q);
           else
