@@ -137,6 +137,9 @@ struct mithra_sim {
   // tiles after the threshold has changed to none)
   int list_below = 0;
   int n_sm = 152;
+  // device scratch of the copy-out calls, kept up to kKeptScratch bytes
+  void* scratch = nullptr;
+  size_t scratch_bytes = 0;
   mithra_batch* in_batch = nullptr;  // the batch that steps this sim, if any
   // per-kernel event timing
   bool profiling = false;
@@ -967,13 +970,43 @@ mithra_status sync_status(mithra_sim* s, bool report_lost = false) {
   return MITHRA_OK;
 }
 
+// Device scratch of one call: the simulation's kept buffer up to
+// kKeptScratch bytes (allocating and freeing 1 MB took longer than copying
+// it), above that allocated and freed with the call.  The calls that use it
+// wait for the stream before they return.
+constexpr size_t kKeptScratch = 4u << 20;
+struct Scratch {
+  void* p = nullptr;
+  bool own = false;
+  cudaError_t get(mithra_sim* s, size_t bytes) {
+    if (bytes > kKeptScratch) {
+      own = true;
+      return cudaMalloc(&p, bytes);
+    }
+    if (s->scratch_bytes < bytes) {
+      if (s->scratch) cudaFree(s->scratch);
+      s->scratch = nullptr;
+      s->scratch_bytes = 0;
+      const cudaError_t e = cudaMalloc(&s->scratch, bytes);
+      if (e != cudaSuccess) return e;
+      s->scratch_bytes = bytes;
+    }
+    p = s->scratch;
+    return cudaSuccess;
+  }
+  ~Scratch() {
+    if (own && p) cudaFree(p);
+  }
+};
+
 template <typename T>
 mithra_status copy_field_impl(mithra_sim* s, int what, double* out) {
   PicP<T> pp = make_pic<T>(s);
   pp.plo = static_cast<const LoV4*>(s->PL[s->cur]);
   const int64_t n = ncell_of(&s->g);
-  double* d = nullptr;
-  MCHECK(s, cudaMalloc(&d, sizeof(double) * n));
+  Scratch sc;
+  MCHECK(s, sc.get(s, sizeof(double) * n));
+  double* const d = static_cast<double*>(sc.p);
   const V4<T>* Pn = static_cast<const V4<T>*>(s->P[s->cur]);
   const V4<T>* Po = static_cast<const V4<T>*>(s->P[1 - s->cur]);
   const V4<T>* Dn = static_cast<const V4<T>*>(s->D);
@@ -994,9 +1027,7 @@ mithra_status copy_field_impl(mithra_sim* s, int what, double* out) {
                                             static_cast<const V4<T>*>(s->S), code, d);
   MCHECK(s, cudaGetLastError());
   MCHECK(s, cudaMemcpyAsync(out, d, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
-  mithra_status st = sync_status(s);
-  cudaFree(d);
-  return st;
+  return sync_status(s);
 }
 
 template <typename T>
@@ -1013,8 +1044,9 @@ mithra_status set_field_impl(mithra_sim* s, int what, const double* in) {
   else if (what == MITHRA_RHO) { dst = static_cast<V4<T>*>(s->S); comp = 3; }
   else if (what >= MITHRA_AX_PREV && what <= MITHRA_PHI_PREV) { dst = static_cast<V4<T>*>(s->P[1 - s->cur]); dstlo = Lp; comp = what - MITHRA_AX_PREV; }
   else return fail(s, MITHRA_EINVAL, "field cannot be set (E and B derive from the potentials)");
-  double* d = nullptr;
-  MCHECK(s, cudaMalloc(&d, sizeof(double) * n));
+  Scratch sc;
+  MCHECK(s, sc.get(s, sizeof(double) * n));
+  double* const d = static_cast<double*>(sc.p);
   MCHECK(s, cudaMemcpyAsync(d, in, sizeof(double) * n, cudaMemcpyHostToDevice, s->stream));
   k_insert<T><<<1024, 256, 0, s->stream>>>(n, d, dst, dstlo, comp);
   if (dst == static_cast<V4<T>*>(s->S)) mark_sources_everywhere(s);
@@ -1023,9 +1055,7 @@ mithra_status set_field_impl(mithra_sim* s, int what, const double* in) {
                                                 static_cast<const V4<T>*>(s->P[1 - s->cur]),
                                                 Lc, Lp, static_cast<V4<T>*>(s->D));
   MCHECK(s, cudaGetLastError());
-  mithra_status st = sync_status(s);
-  cudaFree(d);
-  return st;
+  return sync_status(s);
 }
 
 template <typename T>
@@ -1034,10 +1064,10 @@ mithra_status sample_impl(mithra_sim* s, uint32_t mask, const int32_t* ijk, int6
   PicP<T> pp = make_pic<T>(s);
   pp.plo = static_cast<const LoV4*>(s->PL[s->cur]);
   const int m = __builtin_popcount(mask);
-  int* dijk = nullptr;
-  double* dout = nullptr;
-  MCHECK(s, cudaMalloc(&dijk, sizeof(int) * 3 * npts));
-  MCHECK(s, cudaMalloc(&dout, sizeof(double) * m * npts));
+  Scratch sc;
+  MCHECK(s, sc.get(s, sizeof(double) * m * npts + sizeof(int) * 3 * npts));
+  double* const dout = static_cast<double*>(sc.p);
+  int* const dijk = reinterpret_cast<int*>(dout + m * npts);
   MCHECK(s, cudaMemcpyAsync(dijk, ijk, sizeof(int) * 3 * npts, cudaMemcpyHostToDevice, s->stream));
   k_sample<T><<<blocks_for(npts, 128), 128, 0, s->stream>>>(
       pp, static_cast<const V4<T>*>(s->P[s->cur]), static_cast<const V4<T>*>(s->D),
@@ -1045,10 +1075,7 @@ mithra_status sample_impl(mithra_sim* s, uint32_t mask, const int32_t* ijk, int6
   MCHECK(s, cudaGetLastError());
   MCHECK(s, cudaMemcpyAsync(out, dout, sizeof(double) * m * npts, cudaMemcpyDeviceToHost,
                             s->stream));
-  mithra_status st = sync_status(s);
-  cudaFree(dijk);
-  cudaFree(dout);
-  return st;
+  return sync_status(s);
 }
 
 template <typename T>
@@ -1066,36 +1093,41 @@ mithra_status power_impl(mithra_sim* s, int kp, double* p) {
   return sync_status(s);
 }
 
+// x .. uz into dst[0 .. 5], the lost flags into lost (any may be NULL).
 template <typename T, typename U>
-mithra_status copy_particles_impl(mithra_sim* s, double* out7) {
+mithra_status copy_particles_impl(mithra_sim* s, double* const dst[6], int32_t* lost) {
   const PicP<T> pp = make_pic<T>(s);
-  double* d = nullptr;
-  MCHECK(s, cudaMalloc(&d, sizeof(double) * 7 * (size_t)s->np));
+  const size_t n = (size_t)s->np;
+  Scratch sc;
+  MCHECK(s, sc.get(s, (6 * sizeof(double) + sizeof(int32_t)) * n));
+  double* const d = static_cast<double*>(sc.p);
+  int* const dl = reinterpret_cast<int*>(d + 6 * n);
   k_copy_out<T, U><<<blocks_for(s->np, 256), 256, 0, s->stream>>>(pp, parts_of<T, U>(s, s->pb),
-                                                                  s->np, d);
+                                                                  s->np, d, dl);
   MCHECK(s, cudaGetLastError());
-  MCHECK(s, cudaMemcpyAsync(out7, d, sizeof(double) * 7 * (size_t)s->np, cudaMemcpyDeviceToHost,
-                            s->stream));
-  mithra_status st = sync_status(s);
-  cudaFree(d);
-  return st;
+  for (int a = 0; a < 6; ++a)
+    if (dst[a])
+      MCHECK(s, cudaMemcpyAsync(dst[a], d + a * n, sizeof(double) * n, cudaMemcpyDeviceToHost,
+                                s->stream));
+  if (lost)
+    MCHECK(s, cudaMemcpyAsync(lost, dl, sizeof(int32_t) * n, cudaMemcpyDeviceToHost, s->stream));
+  return sync_status(s);
 }
 
 template <typename T, typename U>
 mithra_status bunch_stats_impl(mithra_sim* s, double kb, double* out14) {
   const PicP<T> pp = make_pic<T>(s);
   const int nb = (int)std::min<long long>(blocks_for(s->np, 256), 1024);
-  double* d = nullptr;
-  MCHECK(s, cudaMalloc(&d, sizeof(double) * ((size_t)nb * kBunchSums + 14)));
+  Scratch sc;
+  MCHECK(s, sc.get(s, sizeof(double) * ((size_t)nb * kBunchSums + 14)));
+  double* const d = static_cast<double*>(sc.p);
   k_bunch_partial<T, U><<<nb, 256, 0, s->stream>>>(pp, parts_of<T, U>(s, s->pb), s->np, kb, d);
   k_bunch_final<<<1, 32, 0, s->stream>>>(d, nb, d + (size_t)nb * kBunchSums);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(out14, d + (size_t)nb * kBunchSums, sizeof(double) * 14,
                         cudaMemcpyDeviceToHost, s->stream);
-  mithra_status st = e == cudaSuccess ? sync_status(s) : cuda_fail(s, e, "bunch statistics");
-  cudaFree(d);
-  return st;
+  return e == cudaSuccess ? sync_status(s) : cuda_fail(s, e, "bunch statistics");
 }
 
 void free_spectrum(mithra_sim* s) {
@@ -1120,7 +1152,7 @@ void free_all(mithra_sim* s) {
   void* ptrs[] = {s->P[0], s->P[1], s->PL[0], s->PL[1], s->D, s->S, s->pbuf[0], s->pbuf[1], s->perm, s->key, s->rank, s->count[0],
                   s->count[1] != s->count[0] ? s->count[1] : nullptr, s->offset, s->tiles, s->units, s->dirty, s->scan_part, s->dstate, s->d_scalar, s->d_power_rec,
                   s->d_spec_omega, s->d_spec_acc, s->d_spec_out, s->d_spec_samples,
-                  s->d_bunch_rec, s->d_bunch_part};
+                  s->d_bunch_rec, s->d_bunch_part, s->scratch};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (s->h_mirror) cudaFreeHost(s->h_mirror);
@@ -1750,17 +1782,12 @@ mithra_status mithra_copy_particles(mithra_sim* s, double* x, double* y, double*
                                     double* uy, double* uz, int32_t* lost, int64_t* n_lost) {
   if (!s) return fail(nullptr, MITHRA_EINVAL, "sim is NULL");
   if (s->np > 0 && (x || y || z || ux || uy || uz || lost)) {
-    std::vector<double> buf((size_t)s->np * 7);
+    double* const dst[6] = {x, y, z, ux, uy, uz};
     mithra_status st = with_types(s->prec, [&](auto t, auto u) {
       TYPES_OF(t, u);
-      return copy_particles_impl<T, U>(s, buf.data());
+      return copy_particles_impl<T, U>(s, dst, lost);
     });
     if (st != MITHRA_OK) return st;
-    double* dst[6] = {x, y, z, ux, uy, uz};
-    for (int a = 0; a < 6; ++a)
-      if (dst[a]) std::memcpy(dst[a], buf.data() + (size_t)a * s->np, sizeof(double) * s->np);
-    if (lost)
-      for (int64_t q = 0; q < s->np; ++q) lost[q] = buf[(size_t)6 * s->np + q] != 0.0 ? 1 : 0;
   }
   if (n_lost) {
     StepState st;

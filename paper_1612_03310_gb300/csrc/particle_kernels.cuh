@@ -983,21 +983,22 @@ __global__ void k_advance(StepState* __restrict__ st, int c) {
   st->src_all[c] = 0;
 }
 
-// Copy-out in the original particle order: FP64 positions from (cell, f).
+// Copy-out in the original particle order: FP64 positions from (cell, f),
+// momenta, and the lost flags.
 template <typename T, typename U>
-__global__ void k_copy_out(PicP<T> p, Parts<T, U> P, long long np, double* __restrict__ out) {
+__global__ void k_copy_out(PicP<T> p, Parts<T, U> P, long long np, double* __restrict__ out,
+                           int* __restrict__ lost) {
   const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (q >= np) return;
   const long long d = P.id[q];
   const int cell = P.cell[q];
-  double x = 0, y = 0, z = 0, lost = 1.0;
+  double x = 0, y = 0, z = 0;
   if (cell >= 0) {
     int i, j, k;
-  decode_cell(p, cell, &i, &j, &k);
+    decode_cell(p, cell, &i, &j, &k);
     x = p.x0 + ((double)i + (double)P.fx[q]) * p.dxd;
     y = p.y0 + ((double)j + (double)P.fy[q]) * p.dyd;
     z = p.z0 + ((double)k + (double)P.fz[q]) * p.dzd;
-    lost = 0.0;
   }
   out[0 * np + d] = x;
   out[1 * np + d] = y;
@@ -1005,7 +1006,7 @@ __global__ void k_copy_out(PicP<T> p, Parts<T, U> P, long long np, double* __res
   out[3 * np + d] = u_dbl(P.ux[q]);
   out[4 * np + d] = u_dbl(P.uy[q]);
   out[5 * np + d] = u_dbl(P.uz[q]);
-  out[6 * np + d] = lost;
+  lost[d] = cell < 0 ? 1 : 0;
 }
 
 }  // namespace mithra
