@@ -188,3 +188,28 @@ def test_update_with_its_boundary(M, orc, prec, shape):  # noqa: F811
                 ref = oracle_fields(o)[nm]
                 tol = 1e-12 if prec == "P64" else 1e-5
                 assert np.abs(sim.copy_field(nm) - ref).max() <= tol * np.abs(ref).max(), nm
+
+
+def test_fused_batch_members_without_particles(M):  # noqa: F811
+    # members without particles list no units, among more members than one
+    # launch of the particle step takes
+    pairs = []
+    for k in range(33):
+        g = dict(inputs.random_grid(100 + k, 16, 16, 16 + k % 5), boundary=1)
+        P = inputs.random_particles(200 + k, g, 100 * (k % 3), u_scale=0.2) if k % 3 else None
+        pairs.append([M.Simulation(g, None, P, precision=M.P32_U64) for _ in range(2)])
+    with M.Batch() as b:
+        b.set_mode(True)
+        for s, _ in pairs:
+            b.add(s)
+        b.step(4)
+        assert b.fused()
+        b.sync()
+        for s, alone in pairs:
+            alone.step(4)
+            for nm in ("Ay", "Ex", "rho"):
+                a, c = s.copy_field(nm), alone.copy_field(nm)
+                assert np.abs(a - c).max() <= 1e-5 * np.abs(c).max(), nm
+    for s, alone in pairs:
+        s.close()
+        alone.close()
