@@ -1318,7 +1318,9 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
   cudaMemsetAsync(s->S, 0, field_bytes, s->stream);
   for (int* c : s->count) cudaMemsetAsync(c, 0, sizeof(int) * (size_t)(s->nkeys + 2), s->stream);
   cudaMemsetAsync(s->dstate, 0, sizeof(StepState), s->stream);
-  cudaMemsetAsync(s->units, 0, sizeof(int4), s->stream);  // no unit listed
+  // no unit listed and no lost particle's slot, until the first re-sort
+  cudaMemsetAsync(s->units, 0, sizeof(int4), s->stream);
+  cudaMemsetAsync(s->offset, 0, sizeof(int) * (size_t)(s->nkeys + 2), s->stream);
   cudaMemsetAsync(s->dirty, 0, 8 * (size_t)s->dirty_words, s->stream);
   mark_sources_everywhere(s);
   {
