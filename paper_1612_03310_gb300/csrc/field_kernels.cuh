@@ -341,6 +341,10 @@ __global__ void __launch_bounds__(256) k_mur_boundary(StencilP<T> p,
                                                       LoV4* __restrict__ nxtlo,
                                                       V4<T>* __restrict__ D,
                                                       V4<T>* __restrict__ src) {
+  // the ring form's CTAs may be placed as soon as every block here has started
+  // (128 x 128 x 1024 cells, step: compensated 430 to 427.5 us, plain 363.5 to
+  // 361.4; 256 x 256 x 2048 3097 to 3095)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   int i, j, k;
   if (kRest ? !rest_vertex(p.nx, p.ny, p.nz, &i, &j, &k)
             : !boundary_vertex(p.nx, p.ny, p.nz, &i, &j, &k))
@@ -1069,6 +1073,9 @@ __global__ void __launch_bounds__(kRThreads, 4) k_potential_ring(
     refill(0);
     ab = vadd<true>(am, b0);
   }
+  // k_mur_boundary, beside which this kernel starts, has read the increments
+  // and sources that the stores below change
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const bool src_every = p.dirty == nullptr || *p.src_all != 0;
   const int trow = (j >> 3) * p.ntx + (i >> 3), ntxy = p.ntx * p.nty;
   long long c = (long long)kb * p.nxy + (long long)j * p.nx + i;

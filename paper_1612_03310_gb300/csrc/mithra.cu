@@ -729,9 +729,22 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
                                        : (fused ? k_potential_ring<kRingAsync, true>
                                                 : k_potential_ring<kRingAsync, false>);
           grd.z = (s->g.nz + rl - 1) / rl;
-          kern<<<grd, kRThreads, ring_smem_bytes(lo), s->stream>>>(
-              s->tm[s->cur], s->tm_lo[s->cur], s->tm_col_d, sp, L0, P1, L1, Dn, S, rl,
-              &s->dstate->err);
+          // a programmatic dependent of the boundary kernel: its CTAs load
+          // their first planes while that one's last wave runs
+          cudaLaunchConfig_t cfg = {};
+          cfg.gridDim = grd;
+          cfg.blockDim = dim3(kRThreads);
+          cfg.dynamicSmemBytes = ring_smem_bytes(lo);
+          cfg.stream = s->stream;
+          cudaLaunchAttribute attr[1];
+          attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+          attr[0].val.programmaticStreamSerializationAllowed = 1;
+          cfg.attrs = attr;
+          cfg.numAttrs = 1;
+          const cudaError_t le =
+              cudaLaunchKernelEx(&cfg, kern, s->tm[s->cur], s->tm_lo[s->cur], s->tm_col_d, sp, L0,
+                                 P1, L1, Dn, S, rl, &s->dstate->err);
+          if (le != cudaSuccess) return cuda_fail(s, le, "potential update launch");
         }
       }
       if (rl > 0) {
