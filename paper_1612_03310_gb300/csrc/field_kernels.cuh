@@ -333,14 +333,14 @@ __device__ __forceinline__ void mur_vertex(const StencilP<T>& p, const V4<T>* __
 // With kRest, only the vertices of rest_vertex (1-D launch of rest_count
 // threads).  kTerms: the interior update is the z-marching form, whose
 // arithmetic D_q^+ is recomputed with.
+// The compensated rest, 68 registers, is held to 64 (4 bytes of spill) for
+// four blocks an SM: it waits for memory at a third of its rate (step of 256 x
+// 256 x 2048 cells 3095 to 3090 us, of 128 x 128 x 1024 427.3 to 426.3).
 template <bool kLo, typename T, bool kRest = false, bool kTerms = false>
-__global__ void __launch_bounds__(256) k_mur_boundary(StencilP<T> p,
-                                                      const V4<T>* __restrict__ cur,
-                                                      const LoV4* __restrict__ curlo,
-                                                      V4<T>* __restrict__ nxt,
-                                                      LoV4* __restrict__ nxtlo,
-                                                      V4<T>* __restrict__ D,
-                                                      V4<T>* __restrict__ src) {
+__global__ void __launch_bounds__(256, kRest && kLo && sizeof(T) == 4 ? 4 : 0)
+    k_mur_boundary(StencilP<T> p, const V4<T>* __restrict__ cur, const LoV4* __restrict__ curlo,
+                   V4<T>* __restrict__ nxt, LoV4* __restrict__ nxtlo, V4<T>* __restrict__ D,
+                   V4<T>* __restrict__ src) {
   // the ring form's CTAs may be placed as soon as every block here has started
   // (128 x 128 x 1024 cells, step: compensated 430 to 427.5 us, plain 363.5 to
   // 361.4; 256 x 256 x 2048 3097 to 3095)
