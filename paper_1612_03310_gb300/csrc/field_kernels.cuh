@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(256, kRest && kLo && sizeof(T) == 4 ? 4 : 0)
   // the ring form's CTAs may be placed as soon as every block here has started
   // (128 x 128 x 1024 cells, step: compensated 430 to 427.5 us, plain 363.5 to
   // 361.4; 256 x 256 x 2048 3097 to 3095)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_dep_launch();
   int i, j, k;
   if (kRest ? !rest_vertex(p.nx, p.ny, p.nz, &i, &j, &k)
             : !boundary_vertex(p.nx, p.ny, p.nz, &i, &j, &k))
@@ -1015,6 +1015,8 @@ __global__ void __launch_bounds__(kRThreads, 4) k_potential_ring(
       cp_async_mbar_arrive(&full[s]);
     }
   };
+  // (its plain loads go through L1 and wait at once)
+  if (kLo == kRingAsync) grid_dep_wait();
   for (int q = 0; q < kRStages && q < nplanes; ++q) issue(q);
 
   const bool xb = kMur && (i == 0 || (i == p.nx - 1 && xhi_fused(p.nx)));
@@ -1075,7 +1077,7 @@ __global__ void __launch_bounds__(kRThreads, 4) k_potential_ring(
   }
   // k_mur_boundary, beside which this kernel starts, has read the increments
   // and sources that the stores below change
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (kLo != kRingAsync) grid_dep_wait();
   const bool src_every = p.dirty == nullptr || *p.src_all != 0;
   const int trow = (j >> 3) * p.ntx + (i >> 3), ntxy = p.ntx * p.nty;
   long long c = (long long)kb * p.nxy + (long long)j * p.nx + i;
