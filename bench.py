@@ -146,23 +146,34 @@ class ClockSampler:
 
 # kernels behind one timed scope of the library's profiler: the potential
 # update is the Mur boundary kernel plus the interior kernel, the re-sort scan
-# two passes
-KERNELS_PER_SCOPE = {"potential_step": 2, "scan_counts": 2}
+# two passes, the particle step the dense and the sparse tiles.  A smaller grid
+# takes as little as one kernel for the whole re-sort, one for every tile and
+# one for the update with its boundary.
+KERNELS_PER_SCOPE = {"potential_step": 2, "scan_counts": 2, "push": 2}
+SMALL_GRID_KEYS = 16 * 3 * 152  # tiles, 16 per persistent CTA
+
+
+def kernels_of(scope: str, n: int, grid: dict) -> int:
+    """Kernels launched by n occurrences of a timed scope, at least."""
+    keys = ((grid["nx"] + 7) // 8) * ((grid["ny"] + 7) // 8) * ((grid["nz"] + 7) // 8)
+    if keys > SMALL_GRID_KEYS:
+        return n * KERNELS_PER_SCOPE.get(scope, 1)
+    return 0 if scope == "slot_map" else n
 
 
 PRECISIONS = {"p32": "P32", "p32_u64": "P32_U64", "p32_c": "P32_C", "p64": "P64"}
 
-# DRAM bytes (read + write) per launch from one ncu capture (--set full, the
+# DRAM bytes (read + write) per launch from one ncu capture (the
 # c2 step in the bench's launch configuration) of the kernels as they are
 # now, by (timed scope, precision, workload); a kernel changed since its
 # capture must leave this table
 NCU_TRAFFIC = {
-    # k_mur_boundary<1, float, 1, 1> + k_potential_zloop_mur1<1, float>
-    ("potential_step", "p32_u64", "c2"): 35241728 + 187392 + 725083904 + 634589184,
+    # k_mur_boundary<1, float, 1, 1> + k_potential_ring<1, 1>
+    ("potential_step", "p32_u64", "c2"): 35241728 + 145152 + 735498496 + 629447424,
     # k_push_tiled<0, float, FF2, 1, 0>
     ("push", "p32_u64", "c2"): None,
-    # k_mur_boundary<0, float, 1, 1> + k_potential_zloop_mur1<0, float>
-    ("potential_step", "p32", "c2"): 28195072 + 39680 + 589268224 + 498427136,
+    # k_mur_boundary<0, float, 1, 1> + k_potential_ring<0, 1>
+    ("potential_step", "p32", "c2"): 28195072 + 33280 + 592309760 + 496057600,
     # k_push_tiled<0, float, float, 0, 0>
     ("push", "p32", "c2"): None,
 }
@@ -347,7 +358,7 @@ def run_gpu(args, rank, world):
                                       for t in rec.get("trials", [])],
                grid=g, n_lost=parts["n_lost"], power_last=float(power[-1, 0]),
                source_reads=src_reads,
-               launches=sum(n * KERNELS_PER_SCOPE.get(k, 1) for k, (_, n) in kt.items()))
+               launches=sum(kernels_of(k, n, g) for k, (_, n) in kt.items()))
 
     # the other precision forms on the same workload, shorter: P64 (plain
     # FP64) and P32_U64 (compensated FP32 levels, FP64 momenta: the form that
