@@ -898,6 +898,11 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         mark_sources_everywhere(s);  // this form marks no tiles
       }
     }
+    // the bunch record reads every particle, the sparse tiles' too
+    if (branch) {
+      cudaEventRecord(s->ev_join, s->side);
+      cudaStreamWaitEvent(s->stream, s->ev_join, 0);
+    }
     if (s->bunch_every > 0) {
       ProfScope ps(s, K_SPECTRUM);
       const int nb = (int)std::min<long long>(blocks_for(s->np, 256), 1024);
@@ -905,10 +910,6 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
                                                         s->dstate, s->bunch_first, s->bunch_every);
       k_bunch_final<<<1, 32, 0, s->stream>>>(s->d_bunch_part, nb, s->d_bunch_rec, s->dstate,
                                              s->bunch_first, s->bunch_every, s->bunch_cap);
-    }
-    if (branch) {
-      cudaEventRecord(s->ev_join, s->side);
-      cudaStreamWaitEvent(s->stream, s->ev_join, 0);
     }
     if (defer && !s->profiling) {
       s->resort_pending = true;

@@ -213,3 +213,28 @@ def test_fused_batch_members_without_particles(M):  # noqa: F811
     for s, alone in pairs:
         s.close()
         alone.close()
+
+
+@pytest.mark.parametrize("prec,tol", [("P64", 1e-11), ("P32_U64", 1e-7)])
+def test_bunch_record_waits_for_the_sparse_tiles(M, prec, tol):  # noqa: F811
+    # every tile sparse, so that all particles are pushed by the kernel beside
+    # the tiled one: each step's record holds the state after that step, as
+    # bunch_stats gives it.  The two differ by the order of the field's atomics
+    # only (weak charges); a step moves the means of these 2e5 particles by
+    # some 0.3 c dt / sqrt(2e5), 2e-5 of the spreads
+    g = dict(inputs.random_grid(121, 64, 64, 64), boundary=1)
+    P = dict(inputs.random_particles(122, g, 200000, u_scale=0.3), q_macro=-1e-18)
+    with M.Simulation(g, None, P, precision=getattr(M, prec)) as sim, \
+            M.Simulation(g, None, P, precision=getattr(M, prec)) as alone:
+        sim.set_tuning(push_sparse_below=1 << 30)
+        sim.set_bunch_sampling(1.0e3, 1, 12)
+        sim.step(12)
+        rec = sim.read_bunch()
+        assert list(rec[:, 0]) == list(range(1, 13))
+        for r in rec:
+            alone.step(1)
+            ref = alone.bunch_stats(1.0e3)
+            spread = ref[6:12]
+            assert (np.abs(r[1:7] - ref[:6]) <= tol * spread).all(), (r[0], r[1:7] - ref[:6])
+            assert (np.abs(r[7:13] - spread) <= tol * spread).all(), (r[0], r[7:13] - spread)
+            assert r[14] == ref[13]
