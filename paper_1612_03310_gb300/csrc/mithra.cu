@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <type_traits>
@@ -137,9 +138,11 @@ struct mithra_sim {
   // tiles after the threshold has changed to none)
   int list_below = 0;
   int n_sm = 152;
-  // device scratch of the copy-out calls, kept up to kKeptScratch bytes
+  // device scratch of the copy-out calls, kept up to kKeptScratch bytes; one
+  // call at a time has it (scratch_mu)
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
+  std::mutex scratch_mu;
   mithra_batch* in_batch = nullptr;  // the batch that steps this sim, if any
   // per-kernel event timing
   bool profiling = false;
@@ -987,14 +990,17 @@ mithra_status sync_status(mithra_sim* s, bool report_lost = false) {
 
 // Device scratch of one call: the simulation's kept buffer up to
 // kKeptScratch bytes (allocating and freeing 1 MB took longer than copying
-// it), above that allocated and freed with the call.  The calls that use it
-// wait for the stream before they return.
+// it); above that, or while another thread's call has the kept buffer,
+// allocated and freed with the call.  The calls that use it wait for the
+// stream before they return.
 constexpr size_t kKeptScratch = 4u << 20;
 struct Scratch {
   void* p = nullptr;
   bool own = false;
+  std::unique_lock<std::mutex> kept;  // held while p is the kept buffer
   cudaError_t get(mithra_sim* s, size_t bytes) {
-    if (bytes > kKeptScratch) {
+    if (bytes <= kKeptScratch) kept = std::unique_lock<std::mutex>(s->scratch_mu, std::try_to_lock);
+    if (!kept.owns_lock()) {
       own = true;
       return cudaMalloc(&p, bytes);
     }

@@ -3,6 +3,8 @@ the potential update, at the sizes
 where they can go wrong: tiles of exactly one, a whole number and one more
 than a whole number of units, key counts around the scans' block sizes, the
 sparse tiles' kernel beside the units, an empty bunch; against the oracle."""
+from concurrent.futures import ThreadPoolExecutor
+
 import numpy as np
 import pytest
 
@@ -238,3 +240,23 @@ def test_bunch_record_waits_for_the_sparse_tiles(M, prec, tol):  # noqa: F811
             assert (np.abs(r[1:7] - ref[:6]) <= tol * spread).all(), (r[0], r[1:7] - ref[:6])
             assert (np.abs(r[7:13] - spread) <= tol * spread).all(), (r[0], r[7:13] - spread)
             assert r[14] == ref[13]
+
+
+def test_copy_out_from_several_threads(M):  # noqa: F811
+    # calls of several threads on one simulation, each with scratch of its
+    # own: fields of 0.25 MB (the kept scratch), particles, samples, and at
+    # (40, 40, 400) a field above the kept scratch's 4 MB
+    for shape in ((32, 32, 32), (40, 40, 400)):
+        g = dict(inputs.random_grid(131, *shape), boundary=1)
+        P = inputs.random_particles(132, g, 20000, u_scale=0.2)
+        ijk = np.random.default_rng(1).integers(1, 30, (3000, 3))
+        with M.Simulation(g, None, P, precision=M.P64) as sim:
+            sim.step(6)
+            calls = [lambda nm=nm: sim.copy_field(nm) for nm in ("Ex", "phi", "rho")] + [
+                lambda: sim.copy_particles()["z"], lambda: sim.copy_particles()["uy"],
+                lambda: sim.sample_fields(["Ey", "Az"], ijk)]
+            ref = [f() for f in calls]
+            with ThreadPoolExecutor(len(calls)) as pool:
+                runs = [pool.submit(lambda f=f, r=r: [np.array_equal(f(), r) for _ in range(40)])
+                        for f, r in zip(calls, ref)]
+                assert all(all(r.result()) for r in runs)
