@@ -155,7 +155,8 @@ __global__ void __launch_bounds__(256) kb_power(const BatchMember<T, U>* __restr
 // (tile_push.cuh): persistent CTAs take every member's units from one
 // counter (k_push_sparse strides over their sparse tiles); kb_tile_prefix
 // numbers both member after member (from the lists the last re-sort left)
-// and clears the counter.
+// and clears the counter.  all: no k_push_sparse follows, the sparse tiles
+// are numbered among the units (after each member's).
 // One block a group of kPushGroup members, whose part of `prefs` holds Mg + 1
 // entries of each prefix, then the counter (prefs_of).
 __host__ __device__ inline int* prefs_of(int* prefs, int group) {
@@ -163,14 +164,17 @@ __host__ __device__ inline int* prefs_of(int* prefs, int group) {
 }
 template <typename T, typename U>
 __global__ void __launch_bounds__(32) kb_tile_prefix(const BatchMember<T, U>* __restrict__ mem,
-                                                     int M, int* __restrict__ prefs) {
+                                                     int M, int* __restrict__ prefs, bool all) {
   static_assert(kPushGroup <= 32, "a warp scans a group");
   const int g0 = blockIdx.x * kPushGroup, Mg = min(kPushGroup, M - g0);
   int* pref = prefs_of(prefs, blockIdx.x);
   int* spref = pref + Mg + 1;
   const int m = threadIdx.x;
   Pair v = 0;
-  if (m < Mg) v = pair_of(mem[g0 + m].units[0].x, mem[g0 + m].st->n_sparse);
+  if (m < Mg) {
+    const int4 n = mem[g0 + m].units[0];
+    v = all ? pair_of(n.x + n.z, 0) : pair_of(n.x, n.z);
+  }
   for (int o = 1; o < 32; o <<= 1) {
     const Pair u = __shfl_up_sync(0xffffffffu, v, o);
     if (m >= o) v += u;

@@ -134,9 +134,6 @@ struct mithra_sim {
   int push_max_per_sm = 1;
   int push_ctas_per_sm = 0;
   int push_sparse_below = 0;  // tiles with fewer particles take the per-warp path
-  // threshold of the scan that built the lists in use (they may hold sparse
-  // tiles after the threshold has changed to none)
-  int list_below = 0;
   int n_sm = 152;
   // device scratch of the copy-out calls, kept up to kKeptScratch bytes; one
   // call at a time has it (scratch_mu)
@@ -516,10 +513,6 @@ int sparse_below(const mithra_sim* s) {
   return s->prec == MITHRA_P64 ? 64 : 32;
 }
 
-// Whether a step's lists can hold sparse tiles: the lists in use at the
-// launch or capture, or those of the re-sorts that follow.
-bool may_be_sparse(const mithra_sim* s) { return s->list_below > 0 || sparse_below(s) > 0; }
-
 // Blocks of the sparse tiles' kernel: eight a multiprocessor (32 warps), so
 // that the device takes some 5000 sparse tiles at once.
 unsigned sparse_grid(int n_sm) { return 8u * n_sm; }
@@ -532,7 +525,7 @@ void launch_scan(mithra_sim* s, int advance, int parity, cudaStream_t q = nullpt
   int* const cnt = s->count[parity];
   int* const next = s->count[1 - parity];
   const int nb = (s->nkeys + 1 + kScanBlock - 1) / kScanBlock;
-  const int below = s->list_below = sparse_below(s);
+  const int below = sparse_below(s);
   const int chunk = unit_chunk(totals_beside(s).np, s->push_grid);
   k_scan_partials<kRestored><<<nb, kScanBlock, 0, q>>>(cnt, s->offset, s->nkeys,
                                                        below, chunk, s->scan_part);
@@ -643,14 +636,13 @@ bool small_resort(const mithra_sim* s) { return s->count[0] != s->count[1]; }
 // grids of few tiles.
 void launch_resort(mithra_sim* s, int parity, cudaStream_t q) {
   if (small_resort(s)) {
-    s->list_below = sparse_below(s);
     // the scan's scope holds the whole re-sort, the slot map's is empty
     { ProfScope none(s, K_SLOT_MAP); }
     ProfScope ps(s, K_SCAN);
     const unsigned nb = std::min<unsigned>(blocks_for(s->np, 4 * kSmallThreads), 2 * s->n_sm);
     k_resort_small<<<nb, kSmallThreads, 0, q>>>(
         s->count[parity], s->count[1 - parity], s->offset, s->tiles, s->units, s->nkeys,
-        s->list_below, unit_chunk(totals_beside(s).np, s->push_grid), s->dstate, s->np, s->key,
+        sparse_below(s), unit_chunk(totals_beside(s).np, s->push_grid), s->dstate, s->np, s->key,
         s->rank, s->perm);
     return;
   }
@@ -813,7 +805,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
   // the sparse tiles' kernel and the plane diagnostics run beside the tiled
   // particle step; with per-kernel timing every kernel stays on the
   // simulation's stream
-  const bool sparse = s->np > 0 && s->push_variant == 1 && s->have_tm && may_be_sparse(s);
+  const bool sparse = s->np > 0 && s->push_variant == 1 && s->have_tm && sparse_below(s) > 0;
   const bool branch = !s->profiling && (s->power_cap > 0 || s->spec_nf > 0 || sparse);
   cudaStream_t dq = s->stream;
   if (branch) {
@@ -863,6 +855,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         PushParams<T, U, false> prm;
         prm.tm_pn = s->tm_box[1 - s->cur];
         prm.tm_d = s->tm_box_d;
+        prm.all = sparse ? 0 : 1;
         PushArgs<T, U>& pa = prm.args;
         pa.p = pp;
         pa.st = s->dstate;
@@ -2294,10 +2287,7 @@ mithra_status capture_fused_typed(mithra_batch* b) {
                      : (lo ? k_push_sparse<false, T, U, kAnyLo, true>
                            : k_push_sparse<false, T, U, false, true>);
   bool sparse = false;
-  for (mithra_sim* s : b->sims) {
-    sparse = sparse || may_be_sparse(s);
-    s->list_below = sparse_below(s);  // the captured scans'
-  }
+  for (const mithra_sim* s : b->sims) sparse = sparse || sparse_below(s) > 0;
   if (cudaFuncSetAttribute(kpush, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
       cudaSuccess)
     return bfail(b, MITHRA_ECUDA, "batched particle step: shared memory attribute");
@@ -2323,7 +2313,8 @@ mithra_status capture_fused_typed(mithra_batch* b) {
     cudaStream_t q = b->stream;
     cudaEventRecord(b->ev_branch[0], q);
     cudaStreamWaitEvent(b->branch[0], b->ev_branch[0], 0);
-    kb_tile_prefix<T, U><<<npg, 32, 0, b->branch[0]>>>(mem, M, b->d_pref);
+    kb_tile_prefix<T, U><<<npg, 32, 0, b->branch[0]>>>(mem, M, b->d_pref,
+                                                           !sparse);
     // boundary and potential update, one launch each per group of up to
     // kZGroup members (their arguments in the launch's parameter space);
     // the groups' block numbers start at the group's first member
@@ -2387,6 +2378,7 @@ mithra_status capture_fused_typed(mithra_batch* b) {
       prm.spref = prm.pref + Mg + 1;
       prm.work = const_cast<int*>(prm.spref) + Mg + 1;
       prm.M = Mg;
+      prm.all = sparse ? 0 : 1;
       if (sparse)
         ksparse<<<sparse_grid(b->sims[0]->n_sm), kSparseThreads, 0, side(0)>>>(prm);
     }

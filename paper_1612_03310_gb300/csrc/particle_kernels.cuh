@@ -725,8 +725,8 @@ __host__ __device__ inline int pair_hi(Pair p) { return (int)(unsigned)(p >> 32)
 // A unit is what one CTA of the particle step takes at a time: a tile, or a
 // run of at most `chunk` of its particles' slots, so that a few heavy tiles
 // (a short bunch: 3000 particles a tile in a hundred tiles) spread over the
-// device instead of keeping one CTA each busy.  units[0].x is their number,
-// units[1 + w] = {tile, first slot, end slot, 0}.
+// device instead of keeping one CTA each busy.  units[0] = {units, dense tiles,
+// sparse tiles, 0}, units[1 + w] = {tile, first slot, end slot, 0}.
 //
 // kRestored: the counts come from a restored offset array instead (the lists
 // are rebuilt for this simulation's own chunk and threshold; offset, count
@@ -814,7 +814,7 @@ __device__ __forceinline__ void scan_final_body(const int* count, int* next,
   }
   if (bidx == 0 && threadIdx.x == 0) {
     if (!kRestored) offset[nkeys + 1] = pair_lo(total[0]);
-    units[0] = make_int4(pair_hi(total[0]), 0, 0, 0);
+    units[0] = make_int4(pair_hi(total[0]), pair_lo(total[1]), pair_hi(total[1]), 0);
     st->n_tiles = pair_lo(total[1]);
     st->n_sparse = pair_hi(total[1]);
     st->work = 0;
@@ -951,7 +951,7 @@ __device__ __forceinline__ void resort_small_body(
   }
   if (lists && threadIdx.x == 0) {
     offset[nkeys + 1] = pair_lo(total_cu);
-    units[0] = make_int4(pair_hi(total_cu), 0, 0, 0);
+    units[0] = make_int4(pair_hi(total_cu), pair_lo(total_ds), pair_hi(total_ds), 0);
     st->n_tiles = pair_lo(total_ds);
     st->n_sparse = pair_hi(total_ds);
     st->work = 0;

@@ -226,6 +226,7 @@ struct PushParams<T, U, false> {
   CUtensorMap tm_pn;  // psi^{n+1}, 11^3 boxes
   CUtensorMap tm_d;   // increment, 11^3 boxes
   PushArgs<T, U> args;
+  int all;  // nonzero: no k_push_sparse beside this launch
 };
 
 template <typename T, typename U>
@@ -237,6 +238,7 @@ struct PushParams<T, U, true> {
   const int* spref;  // spref[0 .. M]: sparse tiles before each member
   int* work;         // unit counter
   int M;
+  int all;  // nonzero: no k_push_sparse beside this launch (pref counts both)
 };
 
 // Source-tile flags (StencilP::dirty): the deposits mark the flags of the
@@ -337,23 +339,37 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
       a.rank[q] = bin_rank(a.count, nk);
     }
   };
-  // the units of one simulation's list, then its sparse tiles and lost
-  // tail (each written once; one simulation runs them straight through, a
-  // batch member by member)
-  // units of the launch
+  // units listed in the launch
   auto units = [&]() {
     if constexpr (kBatch) return prm.pref[prm.M];
     else return prm.args.units[0].x;
   };
-  // unit number w of the launch
+  // unit number w of the launch; where no k_push_sparse runs beside it, the
+  // sparse tiles of the lists are units too, after the listed ones: lists
+  // older than the launch's threshold (set between them, or the launch
+  // captured under another) hold some
   auto unit_of = [&](int w) {
-    if (w >= units()) return make_int4(-1, 0, 0, 0);
-    if constexpr (!kBatch) {
-      return prm.args.units[1 + w];
-    } else {
+    // unit w of member mi, past the listed ones (n: the list's header {units,
+    // dense tiles, sparse tiles})
+    auto late = [](const PushArgs<T, U>& a, int4 n, int w, int mi) {
+      const int tile = a.tiles[n.y + (w - n.x)];
+      return make_int4(tile, a.offset[tile], a.offset[tile + 1], mi);
+    };
+    if constexpr (kBatch) {
+      if (w >= prm.pref[prm.M]) return make_int4(-1, 0, 0, 0);
       const int mi = member_of_tile(prm.pref, prm.M, w);
-      const int4 u = prm.m[mi].units[1 + w - prm.pref[mi]];
-      return make_int4(u.x, u.y, u.z, mi);
+      const PushArgs<T, U>& a = prm.m[mi];
+      w -= prm.pref[mi];
+      // (the entry, whose place is in the list either way, asked for with the header)
+      const int4 n = a.units[0], u = a.units[1 + w];
+      if (w < n.x) return make_int4(u.x, u.y, u.z, mi);
+      return late(a, n, w, mi);
+    } else {
+      const PushArgs<T, U>& a = prm.args;
+      const int4 n = a.units[0];
+      if (w < n.x) return a.units[1 + w];
+      if (!prm.all || w - n.x >= n.z) return make_int4(-1, 0, 0, 0);
+      return late(a, n, w, 0);
     }
   };
   auto counter = [&]() {

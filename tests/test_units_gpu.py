@@ -260,3 +260,30 @@ def test_copy_out_from_several_threads(M):  # noqa: F811
                 runs = [pool.submit(lambda f=f, r=r: [np.array_equal(f(), r) for _ in range(40)])
                         for f, r in zip(calls, ref)]
                 assert all(all(r.result()) for r in runs)
+
+
+def test_graph_captured_before_the_sparse_threshold(M, orc):  # noqa: F811
+    # a caller's own graph of two steps, captured while every tile is staged
+    # (no kernel for sparse tiles in it), replayed on lists whose tiles are all
+    # sparse: its first step pushes them too
+    torch = pytest.importorskip("torch")
+    g = inputs.random_grid(141, 32, 24, 24)
+    P = inputs.random_particles(142, g, 2000, u_scale=0.2)
+    und = dict(C1_UND, z_ent_lab=0.0)
+    o = orc.OracleSim(g, und, P)
+    q = torch.cuda.Stream()
+    with M.Simulation(dict(g, boundary=1), und, P, precision=M.P32_U64, stream=q.cuda_stream) as sim:
+        sim.step(2)
+        sim.sync()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=q, capture_error_mode="thread_local"):
+            sim.step(2)
+        sim.set_tuning(push_sparse_below=1 << 30)
+        sim.step(2)
+        with torch.cuda.stream(q):
+            graph.replay()
+        sim.step(3)
+        o.step(9)
+        sim.sync()
+        compare_fields(sim, o, 1e-5, names=["Ex", "Bz", "phi", "Jx", "rho"])
+        compare_particles(sim, o, 2e-5, 1e-5)
