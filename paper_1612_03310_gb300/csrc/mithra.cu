@@ -475,12 +475,17 @@ int plane_run(const mithra_sim* s) {
 // 75 x 413 93 and 83; 64 x 64 x 256 29 and 27; but 32 x 32 x 128 16 and 20, 65
 // x 65 x 256 31 and 39.  Runs of 4, 16 and 64 planes took 246, 235 and 262 us
 // of the first: longer ones part in z from the CTAs that share their halo.
+// Grids of more than 8 x 65535 planes take the longer run that a launch's z
+// dimension holds.
 int ring_run(const mithra_sim* s) {
   if (s->prec == MITHRA_P64 || !s->have_tm || s->stencil_variant != 2) return 0;
   const int cols = (s->g.nx + 31) / 32 * 32, rows = (s->g.ny + 7) / 8 * 8;
   if (10LL * s->g.nx * s->g.ny < 7LL * cols * rows) return 0;
   if (totals_beside(s).planes < 8LL * 2 * s->n_sm) return 0;
-  return s->lz_auto ? 8 : s->lz;
+  if (!s->lz_auto) return s->lz;
+  int lz = 8;
+  while ((s->g.nz + lz - 1) / lz > 65535) lz *= 2;
+  return lz;
 }
 
 // Whether the register z-marching update of a simulation of its own does

@@ -287,3 +287,31 @@ def test_graph_captured_before_the_sparse_threshold(M, orc):  # noqa: F811
         sim.sync()
         compare_fields(sim, o, 1e-5, names=["Ex", "Bz", "phi", "Jx", "rho"])
         compare_particles(sim, o, 2e-5, 1e-5)
+
+
+@pytest.mark.parametrize("prec", ["P32", "P32_U64"])
+def test_more_planes_than_a_launch_has_runs_of_eight(M, prec):  # noqa: F811
+    # above 8 x 65535 planes: two bunches, each in a window of 64 planes whose
+    # vertices agree with a grid of those planes alone (3 steps reach 3 planes)
+    nz, size = 8 * 65535 + 9, 64
+    small = dict(inputs.random_grid(151, 24, 8, size), boundary=1)
+    P = inputs.random_particles(152, dict(small, nz=40), 300, u_scale=0.2)
+    P = dict(P, z=P["z"] + 12 * small["dz"])
+    big = dict(small, nz=nz)
+    windows = (nz // 2, nz - size)
+    z = np.concatenate([P["z"] + k * small["dz"] for k in windows])
+    both = dict({a: np.tile(P[a], 2) for a in ("x", "y", "ux", "uy", "uz")}, z=z, q_macro=P["q_macro"])
+    k, j, i = np.meshgrid(range(8, size - 8), range(1, 7), range(1, 23), indexing="ij")
+    at = np.stack([i.ravel(), j.ravel(), k.ravel()], 1)
+    names = ["Ex", "Bz", "Az", "phi", "Jz", "rho"]
+    with M.Simulation(big, None, both, precision=getattr(M, prec)) as sim, \
+            M.Simulation(small, None, P, precision=getattr(M, prec)) as ref:
+        sim.step(3)
+        sim.sync()
+        ref.step(3)
+        b = ref.sample_fields(names, at)
+        for k0 in windows:
+            a = sim.sample_fields(names, at + np.array([0, 0, k0]))
+            # z of the big grid is rounded to 2^-52 of 31 m, 1e-10 of a cell
+            assert (np.abs(a - b).max(0) <= 1e-5 * np.abs(b).max(0)).all()
+            assert (np.abs(b).max(0) > 0).all()
