@@ -392,9 +392,10 @@ mithra_status mithra_read_spectrum(mithra_sim* sim, double* dW_domega, int64_t* 
  *     0.7 full, with the planes brought to shared memory by TMA, lo parts
  *     included, several in flight.
  *   lz: planes per CTA of the marching forms (0: about two waves of CTAs for
- *     variant 1; for variant 2 8 where the planes come by TMA, else up to 16,
- *     fewer where the grid, or the batch the simulation is in, would leave
- *     multiprocessors without work).
+ *     variant 1; for variant 2 the library's choice at each launch: 8 where the
+ *     planes come by TMA, else up to 16, fewer where the grid, or the batch the
+ *     simulation is in, would leave multiprocessors without work).  A positive
+ *     lz of variant 2 is kept as it is, in a batch too.
  *   push_variant 0: one thread per particle, E and B evaluated at the eight
  *     vertices from global memory; 1: persistent CTAs over 8^3-cell particle
  *     tiles with the potentials, E/B and the deposit block in shared memory.
@@ -408,8 +409,11 @@ mithra_status mithra_read_spectrum(mithra_sim* sim, double* dW_domega, int64_t* 
  *     smaller ones; 1: every tile staged).  Takes effect from the tile list of
  *     the next re-sort.
  * Defaults: stencil_variant 2 with lz 0 (the fastest form of the potential
- * update on every grid timed; mithra_get_tuning shows the run taken), push_variant 1 when the driver provides TMA
- * tensor maps (else 0), push_ctas_per_sm 0, push_sparse_below 0. */
+ * update on every grid timed), push_variant 1 when the driver provides TMA
+ * tensor maps (else 0), push_ctas_per_sm 0, push_sparse_below 0.
+ * mithra_get_tuning returns the choices as set (lz 0 of variant 2 as 0, of
+ * variant 1 as the run it stands for), so that setting them again changes
+ * nothing. */
 typedef struct {
     int32_t stencil_variant;
     int32_t lz;

@@ -119,7 +119,7 @@ struct mithra_sim {
   // potential-update variant: 0 direct, 1 z-marching TMA tiles (needs tm)
   int stencil_variant = 0;
   int lz = 0;  // planes per CTA of the marching forms
-  bool lz_auto = true;  // register form: by the size of the work (plane_run)
+  bool lz_auto = true;  // variant 2, lz 0: by the size of the work (plane_run, ring_run)
   int march_resident = 608;  // marching CTAs resident on the device at once
   bool have_tm = false;
   CUtensorMap tm[2];      // psi buffers, plane boxes of the marching update
@@ -496,12 +496,6 @@ int ring_run(const mithra_sim* s) {
 // a warp with their neighbours.  A fused batch keeps the boundary kernel (64
 // members of 32 x 32 x 128 cells: 212 us a step with it, 217 without).
 bool mur_all(const mithra_sim* s) { return s->g.boundary == 1 && xhi_fused(s->g.nx); }
-
-// Planes per CTA that the single simulation's z-marching update takes.
-int effective_run(const mithra_sim* s) {
-  const int ring = ring_run(s);
-  return ring > 0 ? ring : plane_run(s);
-}
 
 // Tiles below this many particles take the sparse path (0: none): the
 // caller's threshold, or 32 (FP64: 64) on grids of many tiles per CTA, where
@@ -1372,7 +1366,6 @@ mithra_status mithra_create(const mithra_grid* grid, const mithra_undulator* und
       mithra_status r = setup_push_grid<T, U>(s);
       return r == MITHRA_OK ? setup_march<T>(s) : r;
     });
-    s->lz = effective_run(s);
     if (st != MITHRA_OK) {
       std::string msg = s->err;
       return bail(st, msg);
@@ -1877,10 +1870,8 @@ mithra_status mithra_set_tuning(mithra_sim* s, const mithra_tuning* t) {
     return fail(s, MITHRA_EINVAL,
                 "the marching update keeps single-float levels: not with compensated levels");
   s->stencil_variant = t->stencil_variant;
-  // (the run mithra_get_tuning showed, set again, stays the library's choice)
-  s->lz_auto = t->stencil_variant == 2 && (t->lz == 0 || (s->lz_auto && t->lz == s->lz));
-  s->lz = t->lz > 0 ? t->lz
-                    : (s->lz_auto ? effective_run(s) : default_lz(&s->g, s->march_resident));
+  s->lz_auto = t->stencil_variant == 2 && t->lz == 0;
+  s->lz = t->lz > 0 || s->lz_auto ? t->lz : default_lz(&s->g, s->march_resident);
   s->push_variant = t->push_variant;
   s->push_ctas_per_sm = t->push_ctas_per_sm;
   s->push_sparse_below = t->push_sparse_below;

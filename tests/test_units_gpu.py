@@ -315,3 +315,23 @@ def test_more_planes_than_a_launch_has_runs_of_eight(M, prec):  # noqa: F811
             # z of the big grid is rounded to 2^-52 of 31 m, 1e-10 of a cell
             assert (np.abs(a - b).max(0) <= 1e-5 * np.abs(b).max(0)).all()
             assert (np.abs(b).max(0) > 0).all()
+
+
+def test_tuning_set_again_changes_nothing(M):  # noqa: F811
+    # 64 x 64 x 256 cells, where the library's own run is 8 planes alone: the
+    # library's choice stays 0, an explicit 8 stays 8, and settings that leave
+    # lz out leave it alone
+    g = dict(inputs.random_grid(161, 64, 64, 256), boundary=1)
+    with M.Simulation(g, None, None, precision=M.P32) as sim:
+        assert sim.tuning()["lz"] == 0 and sim.tuning()["stencil_variant"] == 2
+        sim.set_tuning(push_sparse_below=1)
+        sim.set_tuning(**sim.tuning())
+        assert sim.tuning()["lz"] == 0 and sim.tuning()["push_sparse_below"] == 1
+        for lz in (8, 16, 1):
+            sim.set_tuning(lz=lz)
+            sim.set_tuning(push_variant=0)
+            assert sim.tuning()["lz"] == lz
+        sim.set_tuning(lz=0)
+        assert sim.tuning()["lz"] == 0
+        sim.set_tuning(stencil_variant=1)
+        assert sim.tuning()["lz"] >= 8
