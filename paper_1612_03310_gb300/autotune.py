@@ -7,12 +7,14 @@ the fastest particle-step choice independently (the two kernels do not share
 knobs), and caches the result per (device, precision, grid, particle count)
 in a JSON file so that later runs of the same shape skip the search.
 
-The candidates: the direct stencil and the two marching stencils (TMA ring,
-registers) with a range of plane runs per CTA; the per-particle push and the tiled push with 1 .. max
-persistent CTAs per SM, then, for the tiled push with the best CTA count, a
-range of sparse-tile thresholds (tiles below it skip the shared-memory
-staging).  A threshold only acts from the next re-sort, so every push
-candidate gets one untimed step before it is timed.
+The candidates: the direct stencil, the marching stencil of variant 1 with a
+range of plane runs per CTA, and that of variant 2 with the library's own
+choice of the run (lz 0) and a range of given ones; the per-particle push and
+the tiled push with 1 .. max persistent CTAs per SM, then, for the tiled push
+with the best CTA count, a range of sparse-tile thresholds (tiles below it
+skip the shared-memory staging; 0, the library's rule, is timed with the CTA
+counts, and 1 stages every tile).  A threshold only acts from the next
+re-sort, so every push candidate gets one untimed step before it is timed.
 """
 from __future__ import annotations
 
@@ -59,9 +61,11 @@ def device_name() -> str:
 
 
 def key_of(grid: dict, n_particles: int, precision: int) -> str:
-    # particle counts are bucketed by powers of two
+    # particle counts are bucketed by powers of two; the version changes when
+    # a choice comes to mean another kernel (v2: no lz 0 of variant 2, and a
+    # sparse threshold of 0 staged every tile)
     nb = max(int(n_particles), 1).bit_length()
-    return (f"v2|{device_name()}|p{precision}|{grid['nx']}x{grid['ny']}x{grid['nz']}|"
+    return (f"v3|{device_name()}|p{precision}|{grid['nx']}x{grid['ny']}x{grid['nz']}|"
             f"n2^{nb}|sub{grid.get('n_sub', 1)}")
 
 
@@ -78,7 +82,7 @@ def stencil_candidates(grid: dict) -> list[dict]:
     for lz in (8, 16, 24, 32, 48, 64, 96, 128):
         if lz <= grid["nz"]:
             out.append(dict(stencil_variant=1, lz=lz))
-    for lz in (4, 8, 16, 32, 64):
+    for lz in (0, 1, 2, 4, 8, 16, 32, 64):  # 0: the library's choice
         if lz <= grid["nz"]:
             out.append(dict(stencil_variant=2, lz=lz))
     return out
@@ -91,7 +95,7 @@ def push_candidates(max_per_sm: int = 3) -> list[dict]:
     return out
 
 
-SPARSE_THRESHOLDS = (16, 32, 64, 128)
+SPARSE_THRESHOLDS = (1, 16, 32, 64, 128)
 
 
 def sparse_candidates(best: dict) -> list[dict]:

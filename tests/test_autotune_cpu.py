@@ -80,3 +80,41 @@ def test_key_buckets_particle_counts():
     assert autotune.key_of(g, 1000, 1) == autotune.key_of(g, 1023, 1)
     assert autotune.key_of(g, 1000, 1) != autotune.key_of(g, 5000, 1)
     assert autotune.key_of(g, 1000, 1) != autotune.key_of(g, 1000, 0)
+
+
+def test_library_choices_are_candidates():
+    # the defaults themselves (lz 0 of variant 2, threshold 0) and their
+    # opposites: one plane a CTA, every tile staged
+    g = inputs.workload("c1")["grid"]
+    st = autotune.stencil_candidates(g)
+    for lz in (0, 1, 2):
+        assert dict(stencil_variant=2, lz=lz) in st
+    pu = autotune.push_candidates(3)
+    assert any(c["push_variant"] == 1 and c["push_sparse_below"] == 0 for c in pu)
+    assert 1 in [c["push_sparse_below"] for c in autotune.sparse_candidates(pu[-1])]
+
+
+def test_default_wins_where_it_is_fastest(fake, monkeypatch):
+    def times(self):
+        t = self.t
+        st = 1.0 if t["stencil_variant"] == 2 and t["lz"] == 0 else 2.0
+        pu = 1.0 if t["push_variant"] == 1 and t["push_sparse_below"] == 0 else 2.0
+        return {"potential_step": (st * 4, 4), "push": (pu * 4, 4)}
+    monkeypatch.setattr(FakeSim, "kernel_times", times)
+    g = inputs.workload("c1")["grid"]
+    best = autotune.tune(g, None, inputs.random_particles(1, g, 100), 1)
+    assert (best["stencil_variant"], best["lz"]) == (2, 0)
+    assert (best["push_variant"], best["push_sparse_below"]) == (1, 0)
+
+
+def test_entries_of_other_choices_are_not_applied(fake):
+    # an entry stored when the same numbers meant other kernels
+    g = inputs.random_grid(0, 64, 64, 256)
+    b = inputs.random_particles(1, g, 1000)
+    key = autotune.key_of(g, 1000, 1)
+    assert not key.startswith("v2|")
+    autotune._store({key.replace(key.split("|")[0], "v2", 1): dict(
+        tuning=dict(stencil_variant=2, lz=16, push_variant=1, push_ctas_per_sm=0,
+                    push_sparse_below=0))})
+    autotune.tune(g, None, b, 1)
+    assert fake.made == 1  # searched anew
