@@ -168,7 +168,7 @@ typedef struct {
  * given, see mithra_make_bunch for Sec. "Electron Bunch Generation"):
  * validates the grid (MITHRA_EUNSTABLE if dt breaks
  * the stability condition, see mithra_check_grid), allocates device memory
- * (mithra_footprint bytes), copies the bunch, sorts it into cell tiles and
+ * (mithra_footprint), copies the bunch, sorts it into cell tiles and
  * deposits rho^{1/2}.  Potentials start at zero at levels -1 and 0, J^0 = 0,
  * the frame clock at t0 = 0.  cuda_stream: a cudaStream_t to order all work
  * on, or NULL for a stream the library creates and owns (pass
@@ -535,8 +535,11 @@ mithra_status mithra_batch_destroy(mithra_batch* batch);
  * stayed bounded up to r_x^2 + r_y^2 = 0.97. */
 mithra_status mithra_check_grid(const mithra_grid* grid);
 
-/* Device bytes mithra_create will allocate for this grid, particle count and
- * precision (used for admission by memory footprint). */
+/* Device bytes that a simulation of this grid, particle count and precision
+ * holds (used for admission by memory footprint): what mithra_create
+ * allocates, and the scratch that the copy-out and field-setting calls keep
+ * from the first of them on (1 to 4 MB: a whole field or all particles, where
+ * they take no more).  Recording diagnostics come on top. */
 mithra_status mithra_footprint(const mithra_grid* grid, int64_t n_particles,
                                mithra_precision precision, int64_t* bytes);
 

@@ -135,7 +135,7 @@ struct mithra_sim {
   int push_ctas_per_sm = 0;
   int push_sparse_below = 0;  // tiles with fewer particles take the per-warp path
   int n_sm = 152;
-  // device scratch of the copy-out calls, kept up to kKeptScratch bytes; one
+  // device scratch of the copy-out calls, kept up to kept_scratch bytes; one
   // call at a time has it (scratch_mu)
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
@@ -243,6 +243,21 @@ mithra_status with_types(int prec, F&& f) {
   using U = std::remove_pointer_t<decltype(u)>
 
 int64_t ncell_of(const mithra_grid* g) { return (int64_t)g->nx * g->ny * g->nz; }
+
+// Bytes of scratch per particle of mithra_copy_particles.
+constexpr size_t kCopyParticle = 6 * sizeof(double) + sizeof(int32_t);
+
+// The most bytes of copy-out scratch that a simulation keeps between calls
+// (allocating and freeing 1 MB took longer than copying it): room for a whole
+// field and for all particles, of either that takes no more than 4 MB, and at
+// least 1 MB.  Part of mithra_footprint.
+size_t kept_scratch(const mithra_grid& g, int64_t np) {
+  constexpr size_t kMost = 4u << 20, kLeast = 1u << 20;
+  size_t b = kLeast;
+  for (const size_t need : {sizeof(double) * (size_t)ncell_of(&g), kCopyParticle * (size_t)np})
+    if (need <= kMost) b = std::max(b, need);
+  return b;
+}
 
 void tiles_of(const mithra_grid* g, int* ntx, int* nty, int* ntz) {
   *ntx = (g->nx + kTile - 1) / kTile;
@@ -981,17 +996,16 @@ mithra_status sync_status(mithra_sim* s, bool report_lost = false) {
 }
 
 // Device scratch of one call: the simulation's kept buffer up to
-// kKeptScratch bytes (allocating and freeing 1 MB took longer than copying
-// it); above that, or while another thread's call has the kept buffer,
-// allocated and freed with the call.  The calls that use it wait for the
-// stream before they return.
-constexpr size_t kKeptScratch = 4u << 20;
+// kept_scratch bytes; above that, or while another thread's call has the kept
+// buffer, allocated and freed with the call.  The calls that use it wait for
+// the stream before they return.
 struct Scratch {
   void* p = nullptr;
   bool own = false;
   std::unique_lock<std::mutex> kept;  // held while p is the kept buffer
   cudaError_t get(mithra_sim* s, size_t bytes) {
-    if (bytes <= kKeptScratch) kept = std::unique_lock<std::mutex>(s->scratch_mu, std::try_to_lock);
+    if (bytes <= kept_scratch(s->g, s->np))
+      kept = std::unique_lock<std::mutex>(s->scratch_mu, std::try_to_lock);
     if (!kept.owns_lock()) {
       own = true;
       return cudaMalloc(&p, bytes);
@@ -1112,7 +1126,7 @@ mithra_status copy_particles_impl(mithra_sim* s, double* const dst[6], int32_t* 
   const PicP<T> pp = make_pic<T>(s);
   const size_t n = (size_t)s->np;
   Scratch sc;
-  MCHECK(s, sc.get(s, (6 * sizeof(double) + sizeof(int32_t)) * n));
+  MCHECK(s, sc.get(s, kCopyParticle * n));
   double* const d = static_cast<double*>(sc.p);
   int* const dl = reinterpret_cast<int*>(d + 6 * n);
   k_copy_out<T, U><<<blocks_for(s->np, 256), 256, 0, s->stream>>>(pp, parts_of<T, U>(s, s->pb),
@@ -1221,6 +1235,7 @@ mithra_status mithra_footprint(const mithra_grid* grid, int64_t n_particles,
   b += 8 * ((nkeys + 3) / 4);                                     // source-tile flags
   b += (nkeys / kScanBlock + 2) * (int64_t)sizeof(int4);         // scan block sums
   b += (int64_t)sizeof(StepState) + (int64_t)sizeof(double);
+  b += (int64_t)kept_scratch(*grid, n_particles);
   *bytes = b;
   return MITHRA_OK;
 }

@@ -161,3 +161,28 @@ def test_boost_from_lab_reproduces_the_workloads(M):
         args.update(bad)
         with pytest.raises(M.MithraError):
             M.boost_from_lab(**args)
+
+
+def test_footprint_counts_the_kept_scratch(M):
+    # a particle more or less on both sides of where all particles (52 bytes
+    # each) stop fitting the 4 MB of scratch that a simulation keeps; the rest
+    # of the footprint grows by the same amount a particle throughout
+    g = dict(inputs.random_grid(0, 8, 8, 8), boundary=1)
+
+    def at(n):
+        return M.footprint(g, n, M.P64)
+    least, most = (1 << 20) // 52, (4 << 20) // 52  # 20164, 80659
+    # the units' list grows by 16 bytes every 256 particles: steps of 256
+    plain = at(10240) - at(10240 - 256)
+    assert at(least // 256 * 256) - at(least // 256 * 256 - 256) == plain
+    assert at(40960) - at(40960 - 256) == plain + 52 * 256
+    assert at(most // 256 * 256) - at(most // 256 * 256 - 256) == plain + 52 * 256
+    over = (most // 256 + 1) * 256  # above: 1 MB kept, as for few particles
+    assert at(over) - at(10240) == (over - 10240) // 256 * plain
+    # a field of 8 bytes a vertex, kept up to 524288 vertices: 64 x 64 x 128
+    # (8 planes more or less are 8 x 8 x 8 / 8 = 64 tiles; the scan's block sums
+    # take another 16 bytes from 1024 tiles on)
+    def field(nz):
+        return M.footprint(dict(g, nx=64, ny=64, nz=nz), 0, M.P64)
+    kept = (field(128) - field(120)) - (field(152) - field(144))
+    assert abs(kept - 8 * 64 * 64 * 8) <= 16
