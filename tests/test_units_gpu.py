@@ -3,6 +3,7 @@ the potential update, at the sizes
 where they can go wrong: tiles of exactly one, a whole number and one more
 than a whole number of units, key counts around the scans' block sizes, the
 sparse tiles' kernel beside the units, an empty bunch; against the oracle."""
+import ctypes as C
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -335,3 +336,36 @@ def test_tuning_set_again_changes_nothing(M):  # noqa: F811
         assert sim.tuning()["lz"] == 0
         sim.set_tuning(stencil_variant=1)
         assert sim.tuning()["lz"] >= 8
+
+
+@pytest.mark.parametrize("shape,n", [((16, 16, 24), 80659), ((16, 16, 24), 80660),
+                                     ((64, 64, 128), 500), ((64, 64, 129), 500)])
+def test_copy_out_parts_and_sizes(M, shape, n):  # noqa: F811
+    # outputs on both sides of what fits the kept scratch (4 MB: 80659
+    # particles, 524288 vertices), in turn on one simulation; any of the
+    # particle arrays NULL leaves the others whole and itself untouched
+    g = dict(inputs.random_grid(171, *shape), boundary=1)
+    P = dict(inputs.random_particles(172, g, n, u_scale=2.0), q_macro=-1e-18)
+    names = ("x", "y", "z", "ux", "uy", "uz")
+    with M.Simulation(g, None, P, precision=M.P64) as sim:
+        sim.step(6)
+        whole = sim.copy_particles()
+        assert 0 < whole["lost"].sum() == whole["n_lost"] < n
+        ex = sim.copy_field("Ex")
+        ijk = np.random.default_rng(2).integers(1, 14, (200, 3))
+        at = sim.sample_fields(["Ex"], ijk)[:, 0]
+        assert np.array_equal(at, ex[ijk[:, 2], ijk[:, 1], ijk[:, 0]])
+        for keep in ([], ["x"], ["uz", "lost"], ["lost"], ["y", "ux"]):
+            out = {a: np.full(n, -7.0) for a in names}
+            lost = np.full(n, -7, np.int32)
+            nl = C.c_int64(-1)
+            ptr = [M._dp(out[a]) if a in keep else None for a in names]
+            lp = lost.ctypes.data_as(C.POINTER(C.c_int32)) if "lost" in keep else None
+            assert M.lib().mithra_copy_particles(sim.h, *ptr, lp, C.byref(nl)) == M.OK
+            assert nl.value == whole["n_lost"]
+            for a in names:
+                assert np.array_equal(out[a], whole[a] if a in keep else np.full(n, -7.0)), a
+            assert np.array_equal(lost, whole["lost"] if lp else np.full(n, -7, np.int32))
+            assert np.array_equal(sim.copy_field("Ex"), ex)
+        again = sim.copy_particles()
+        assert all(np.array_equal(again[a], whole[a]) for a in names + ("lost",))
