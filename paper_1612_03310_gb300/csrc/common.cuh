@@ -170,9 +170,9 @@ struct StepState {
   long long n_lost;     // particles lost so far
   int err;              // bit 0: NaN/Inf in a reduction; bit 1: a bounded wait gave up
   int n_tiles;          // dense tiles listed by the last scan (entries 0 .. n_tiles-1)
-  int work;             // next dense entry of the tile list to hand out
+  int work;             // units handed out beyond each CTA's first
   int n_sparse;         // sparse tiles, listed after the dense ones
-  int work_sparse;      // next sparse entry to hand out
+  int unused;           // keeps the layout of saved snapshots
   // per level parity c: nonzero when sources may sit outside the tiles
   // marked in the parity's flag array (see StencilP::dirty), so that the
   // potential update of parity c reads every vertex's sources

@@ -818,7 +818,6 @@ __device__ __forceinline__ void scan_final_body(const int* count, int* next,
     st->n_tiles = pair_lo(total[1]);
     st->n_sparse = pair_hi(total[1]);
     st->work = 0;
-    st->work_sparse = 0;
     if (advance) st->n += 1;
   }
 }
@@ -955,7 +954,6 @@ __device__ __forceinline__ void resort_small_body(
     st->n_tiles = pair_lo(total_ds);
     st->n_sparse = pair_hi(total_ds);
     st->work = 0;
-    st->work_sparse = 0;
     st->n += 1;
   }
   for (int t = bidx * blockDim.x + threadIdx.x; t <= nkeys; t += nblocks * blockDim.x)
