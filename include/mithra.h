@@ -474,7 +474,7 @@ mithra_status mithra_plane_power_noalloc(const mithra_grid* grid, double gamma0,
  *     of the grid phases one more): the boundary rest, the potential update,
  *     the power sample, the numbering of the members' work units, the
  *     particle step, and the re-sort (one kernel where every member has at
- *     most 4096 tiles, else two scan passes and the slot map), each over a
+ *     most 4095 tiles, else two scan passes and the slot map), each over a
  *     work list that spans all members (flat block lists for the grid phases,
  *     persistent CTAs taking every member's units from one counter for the
  *     particle step), with each member's arguments in the launch's parameter

@@ -17,7 +17,7 @@ __device__ inline void sincos_t(double a, double* s, double* c) { sincos(a, s, c
 // sinh a = m (1 + e^{-a}) / 2 (no cancellation for small a) and
 // cosh a = (e^a + e^{-a}) / 2.
 // For |a| <= 1/2 (ku y of a beam near the axis) the Taylor series, whose next
-// terms are 0.5^10/10! = 3e-10 and 0.5^9/9! / 0.5 = 1e-8.
+// terms are 0.5^10/10! = 3e-10 and, relative to sinh, 0.5^10/11! = 2e-11.
 __device__ inline void coshsinh_t(float a, float* ch, float* sh) {
   if (fabsf(a) <= 0.5f) {
     const float q = a * a;
@@ -37,8 +37,9 @@ __device__ inline void coshsinh_t(float a, float* ch, float* sh) {
   *sh = 0.5f * m * (1.0f + inv);
 }
 // FP64: the Taylor series for |a| <= 1/2 (ku y of a beam near the axis; the
-// next terms are 0.5^18/18! = 6e-22 and 0.5^17/17!), 18 operations on the
-// FP64 pipe, which bounds this form, instead of two library calls.
+// next terms are 0.5^18/18! = 6e-22 and, relative to sinh, 0.5^16/17! =
+// 4e-20), 18 operations on the FP64 pipe, which bounds this form, instead of
+// two library calls.
 __device__ inline void coshsinh_t(double a, double* ch, double* sh) {
   if (fabs(a) <= 0.5) {
     const double q = a * a;
@@ -888,15 +889,16 @@ __global__ void __launch_bounds__(256) k_slot_map(long long np, const int* __res
 }
 
 // The whole re-sort (scan, lists and slot map) of a grid of at most
-// kSmallKeys keys in one launch: every block scans all the counts (16 KB from
-// L2 at most) into offsets in shared memory, then maps its share of the
-// particles; block 0 also writes the offsets, the lists and the step state.
-// The counts of the next step are the other of two arrays, so that clearing
-// it disturbs no block's scan.  What bounds the re-sort of a small grid is
-// launches and latency: by event pairs (some 5 us of each) three kernels took
-// 12 + 6 us and this one 8 on 32 x 32 x 64 cells with 4096 particles (129
-// keys), 13 + 7 and 12 on 64 x 64 x 256 with 262144 (2049 keys); at 6761
-// keys, where each thread walks 14, 13 + 8 and 19, so the line is drawn below.
+// kSmallKeys keys (the tiles and the lost particles' bucket) in one launch:
+// every block scans all the counts (16 KB from L2 at most) into offsets in
+// shared memory, then maps its share of the particles; block 0 also writes
+// the offsets, the lists and the step state.  The counts of the next step are
+// the other of two arrays, so that clearing it disturbs no block's scan.
+// What bounds the re-sort of a small grid is launches and latency: by event
+// pairs (some 5 us of each) three kernels took 12 + 6 us and this one 8 on 32
+// x 32 x 64 cells with 4096 particles (129 keys), 13 + 7 and 12 on 64 x 64 x
+// 256 with 262144 (2049 keys); at 6761 keys, where each thread walks 14, 13 +
+// 8 and 19, so the line is drawn below.
 constexpr int kSmallPer = 8;  // keys a thread
 constexpr int kSmallThreads = 512;
 constexpr int kSmallKeys = kSmallPer * kSmallThreads;

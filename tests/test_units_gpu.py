@@ -369,3 +369,23 @@ def test_copy_out_parts_and_sizes(M, shape, n):  # noqa: F811
             assert np.array_equal(sim.copy_field("Ex"), ex)
         again = sim.copy_particles()
         assert all(np.array_equal(again[a], whole[a]) for a in names + ("lost",))
+
+
+def test_resort_of_the_most_keys_of_one_kernel(M, orc):  # noqa: F811
+    # 9 x 13 x 35 = 4095 tiles and the lost particles' bucket: eight keys a
+    # thread, every one of the 4096 in use; particles in the last tile, and
+    # some that leave the grid through it
+    g = inputs.random_grid(181, 72, 104, 280)
+    P = inputs.random_particles(182, g, 3000, u_scale=0.2)
+    rng = np.random.default_rng(183)
+    h = np.array([g["dx"], g["dy"], g["dz"]])
+    last = np.array([64.0, 96.0, 272.0]) + rng.random((400, 3)) * [4.0, 4.0, 4.5]
+    r = np.array([g["x0"], g["y0"], g["z0"]]) + last * h
+    u = 0.2 * rng.standard_normal((3, 400))
+    u[2, :100] = 3.0
+    P = dict(P, **{a: np.concatenate([P[a], v]) for a, v in
+                   zip(("x", "y", "z", "ux", "uy", "uz"), (*r.T, *u))})
+    check(M, orc, g, dict(C1_UND, z_ent_lab=0.0), P, "P32_U64", (1, 4, 4))
+    o = orc.OracleSim(g, dict(C1_UND, z_ent_lab=0.0), P)
+    o.step(9)
+    assert 50 < o.lost.sum() < 400
