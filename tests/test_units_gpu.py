@@ -389,3 +389,61 @@ def test_resort_of_the_most_keys_of_one_kernel(M, orc):  # noqa: F811
     o = orc.OracleSim(g, dict(C1_UND, z_ent_lab=0.0), P)
     o.step(9)
     assert 50 < o.lost.sum() < 400
+
+
+def kernels_of_a_step(M, g, P, prec, path):  # noqa: F811
+    """Names (mangled) of the kernels that one step launches, from a graph
+    captured of it and never run."""
+    torch = pytest.importorskip("torch")
+    q = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with M.Simulation(g, None, P, precision=getattr(M, prec), stream=q.cuda_stream) as sim:
+        with torch.cuda.graph(graph, stream=q, capture_error_mode="thread_local"):
+            sim.step(1)
+        dot = C.CDLL("libcuda.so.1").cuGraphDebugDotPrint  # verbose: 1
+        assert dot(C.c_void_p(graph.raw_cuda_graph()), str(path).encode(), C.c_uint(1)) == 0
+    return path.read_text()
+
+
+def smooth_levels(g):
+    """Two levels of every component: a constant of order 1 with a hundredth
+    of smooth variation, the second a little later than the first; none of the
+    values are FP32 numbers."""
+    k, j, i = np.meshgrid(np.arange(g["nz"]) / 40.0, np.arange(g["ny"]) / 36.0,
+                          np.arange(g["nx"]) / 44.0, indexing="ij")
+    levels = [np.concatenate([
+        (1.0 / (3 + c) + 0.01 * np.sin(2 * np.pi * (i + 0.7 * j - k + 0.1 * c) + late)).ravel()
+        for c in range(4)]) for late in (0.0, 0.02)]
+    return dict(prev=levels[0], cur=levels[1], src=np.zeros_like(levels[0]))
+
+
+@pytest.mark.parametrize("boundary", [1, 2])
+@pytest.mark.parametrize("shape,lo", [((64, 72, 273), "TMA"), ((129, 40, 155), "cp.async"),
+                                      ((130, 48, 155), "TMA"), ((97, 80, 243), "cp.async"),
+                                      ((127, 57, 155), "cp.async")])
+def test_ring_update_keeps_the_lo_parts(M, orc, boundary, shape, lo, tmp_path):  # noqa: F811
+    # levels near 1 whose second differences are some 1e-4: the hi parts alone
+    # round each level by up to 2^-25 = 3e-8 of it, a wrong lo part is worth as
+    # much, and the right ones (8 more bits) leave 2^-33 = 1.2e-10, a few times
+    # that after four steps' sums (measured 2.9e-10).  The bound lies between,
+    # and plain FP32 has to miss it.  The second-order faces' own terms read hi
+    # parts alone, in every form; what they leave travels a vertex a step, so
+    # that with them the five outermost vertices are left out.
+    g = dict(inputs.random_grid(191, *shape), boundary=boundary)
+    f = smooth_levels(g)
+    # RingLo of the kernel's template: 1 by TMA, 2 by cp.async; 0 plain
+    names = {"P32_C": "k_potential_ringILi%d" % (1 if lo == "TMA" else 2), "P32": "k_potential_ringILi0"}
+    o = orc.OracleSim(g, None, dict(x=[], y=[], z=[], ux=[], uy=[], uz=[]))
+    err = {}
+    for prec in ("P32_C", "P32"):
+        assert names[prec] in kernels_of_a_step(M, g, None, prec, tmp_path / prec)
+        with M.Simulation(g, None, None, precision=getattr(M, prec)) as sim:
+            set_state(sim, o, f)
+            o.step(4)
+            sim.step(4)
+            sim.sync()
+            ref = oracle_fields(o)
+            inner = slice(5, -5) if boundary == 2 else slice(None)
+            err[prec] = max(np.abs(sim.copy_field(nm) - ref[nm])[inner, inner, inner].max()
+                            for nm in ("Ax", "Ay", "Az", "phi"))
+    assert err["P32_C"] <= 2e-9 < 3e-8 < err["P32"], err
