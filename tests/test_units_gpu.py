@@ -447,3 +447,55 @@ def test_ring_update_keeps_the_lo_parts(M, orc, boundary, shape, lo, tmp_path): 
             err[prec] = max(np.abs(sim.copy_field(nm) - ref[nm])[inner, inner, inner].max()
                             for nm in ("Ax", "Ay", "Az", "phi"))
     assert err["P32_C"] <= 2e-9 < 3e-8 < err["P32"], err
+
+
+@pytest.mark.parametrize("prec", ["P32", "P32_U64", "P64"])
+def test_fused_batch_of_sparse_and_dense_members(M, prec):  # noqa: F811
+    # 67 uneven members, three groups of the particle step: in turn mixed lists
+    # (a dense clump in a thin cloud), all sparse, all dense, none sparse with
+    # no particles, and a member whose threshold makes one tile of all dense;
+    # each as its lone run, and as its lone run with every tile staged
+    rng = np.random.default_rng(201)
+    trios, kinds = [], []
+    for k in range(67):
+        kind = k % 5
+        shape = [int(v) for v in rng.integers(16, 34, 3)]
+        g = dict(inputs.random_grid(300 + k, *shape, n_sub=1 + k % 2), boundary=1)
+        n = 0 if kind == 3 else int(rng.integers(200, 900))
+        P = inputs.random_particles(400 + k, g, n, u_scale=0.2) if n else None
+        if kind == 0:  # a third of the particles within a cell or two of a vertex
+            c = {a: P[a][0] + 0.8 * g["d" + a] * rng.random(n // 3) for a in "xyz"}
+            P = dict(P, **{a: np.concatenate([P[a][:-(n // 3)], c[a]]) for a in "xyz"})
+        sims = [M.Simulation(g, None, P, precision=getattr(M, prec)) for _ in range(3)]
+        below = {0: 60, 1: 1 << 30, 2: 1, 3: 60, 4: 25}[kind]
+        for s in sims[:2]:
+            s.set_tuning(push_sparse_below=below)
+        sims[2].set_tuning(push_sparse_below=1)
+        trios.append(sims)
+        kinds.append(kind)
+    tol = 1e-11 if prec == "P64" else 1e-5
+    with M.Batch() as b:
+        b.set_mode(True)
+        for s in trios:
+            b.add(s[0])
+        b.step(6)
+        assert b.fused()
+        b.step(3)
+        b.step(2)
+        b.sync()
+        for k, (inb, alone, staged) in enumerate(trios):
+            for s in (alone, staged):
+                s.step(11)
+                for nm in ("Ay", "Ex", "Jz", "rho"):
+                    a, c = inb.copy_field(nm), s.copy_field(nm)
+                    assert np.linalg.norm(a - c) <= tol * np.linalg.norm(c), (k, kinds[k], nm)
+                if kinds[k] != 3:
+                    a, c = inb.copy_particles(), s.copy_particles()
+                    assert np.array_equal(a["lost"], c["lost"]), k
+                    for nm, d in (("x", "dx"), ("y", "dy"), ("z", "dz")):
+                        assert np.abs(a[nm] - c[nm]).max() <= tol * inb.grid[d], (k, kinds[k], nm)
+                    for nm in ("ux", "uy", "uz"):
+                        assert np.abs(a[nm] - c[nm]).max() <= tol * np.abs(c[nm]).max(), (k, nm)
+    for sims in trios:
+        for s in sims:
+            s.close()
