@@ -522,7 +522,7 @@ bool mur_all(const mithra_sim* s) { return s->g.boundary == 1 && xhi_fused(s->g.
 // particles: 225 us a step staged, 238 at 32, 268 at 128).
 int sparse_below(const mithra_sim* s) {
   if (s->push_variant != 1 || !s->have_tm) return 0;
-  if (s->push_sparse_below > 0) return s->push_sparse_below;
+  if (s->push_sparse_below > 0) return s->push_sparse_below > 1 ? s->push_sparse_below : 0;
   if (s->nkeys < 16 * s->push_grid) return 0;
   return s->prec == MITHRA_P64 ? 64 : 32;
 }

@@ -391,13 +391,15 @@ def test_resort_of_the_most_keys_of_one_kernel(M, orc):  # noqa: F811
     assert 50 < o.lost.sum() < 400
 
 
-def kernels_of_a_step(M, g, P, prec, path):  # noqa: F811
+def kernels_of_a_step(M, g, P, prec, path, **tuning):  # noqa: F811
     """Names (mangled) of the kernels that one step launches, from a graph
     captured of it and never run."""
     torch = pytest.importorskip("torch")
     q = torch.cuda.Stream()
     graph = torch.cuda.CUDAGraph(keep_graph=True)
     with M.Simulation(g, None, P, precision=getattr(M, prec), stream=q.cuda_stream) as sim:
+        if tuning:
+            sim.set_tuning(**tuning)
         with torch.cuda.graph(graph, stream=q, capture_error_mode="thread_local"):
             sim.step(1)
         dot = C.CDLL("libcuda.so.1").cuGraphDebugDotPrint  # verbose: 1
@@ -522,3 +524,11 @@ def test_automatic_sparse_threshold(M, orc, prec, shape, tmp_path):  # noqa: F81
     names = kernels_of_a_step(M, g, P, prec, tmp_path / "step")
     assert ("k_push_sparse" in names) == (tiles >= 16 * per_sm * n_sm)
     check(M, orc, g, None, P, prec, (1, 3))
+
+
+def test_staged_threshold_launches_no_sparse_kernel(M, tmp_path):  # noqa: F811
+    g = dict(inputs.random_grid(221, 32, 24, 24), boundary=1)
+    P = inputs.random_particles(222, g, 500, u_scale=0.2)
+    for below, there in ((0, False), (1, False), (2, True), (1 << 30, True)):
+        names = kernels_of_a_step(M, g, P, "P32", tmp_path / str(below), push_sparse_below=below)
+        assert "k_push_tiled" in names and ("k_push_sparse" in names) == there, below
