@@ -817,16 +817,20 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
     }
   }
   // the sparse tiles' kernel and the plane diagnostics run beside the tiled
-  // particle step; with per-kernel timing every kernel stays on the
-  // simulation's stream
+  // particle step; with per-kernel timing the diagnostics stay on the
+  // simulation's stream, and the particle step's scope holds both its kernels
   const bool sparse = s->np > 0 && s->push_variant == 1 && s->have_tm && sparse_below(s) > 0;
-  const bool branch = !s->profiling && (s->power_cap > 0 || s->spec_nf > 0 || sparse);
-  cudaStream_t dq = s->stream;
-  if (branch) {
+  const bool diag_branch = !s->profiling && (s->power_cap > 0 || s->spec_nf > 0);
+  auto fork = [&]() {
     cudaEventRecord(s->ev_fork, s->stream);
     cudaStreamWaitEvent(s->side, s->ev_fork, 0);
-    dq = s->side;
-  }
+  };
+  auto join = [&]() {
+    cudaEventRecord(s->ev_join, s->side);
+    cudaStreamWaitEvent(s->stream, s->ev_join, 0);
+  };
+  if (diag_branch) fork();
+  cudaStream_t dq = diag_branch ? s->side : s->stream;
   if (s->power_cap > 0) {
     ProfScope ps(s, K_POWER);
     // without particles the two diagnostics run beside each other
@@ -890,8 +894,10 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
         pa.dirty = s->dirty;
         pa.dirty_words = s->dirty_words;
         pa.cur = s->cur;
-        if (sparse)
-          kern_sp<<<sparse_grid(s->n_sm), kSparseThreads, 0, branch ? s->side : s->stream>>>(prm);
+        if (sparse) {
+          if (!diag_branch) fork();
+          kern_sp<<<sparse_grid(s->n_sm), kSparseThreads, 0, s->side>>>(prm);
+        }
         const cudaError_t le = launch_after(s->stream, dim3(s->push_grid), dim3(kPushThreads),
                                             tile_smem_bytes<T, U>(), kern, prm);
         if (le != cudaSuccess) return cuda_fail(s, le, "particle step launch");
@@ -907,11 +913,8 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
                                                              s->rank, &s->dstate->n_lost);
         mark_sources_everywhere(s);  // this form marks no tiles
       }
-    }
-    // the bunch record reads every particle, the sparse tiles' too
-    if (branch) {
-      cudaEventRecord(s->ev_join, s->side);
-      cudaStreamWaitEvent(s->stream, s->ev_join, 0);
+      // before the bunch record too, which reads every particle
+      if (diag_branch || sparse) join();
     }
     if (s->bunch_every > 0) {
       ProfScope ps(s, K_SPECTRUM);
@@ -929,10 +932,7 @@ mithra_status launch_step(mithra_sim* s, bool defer = false) {
     }
     s->pb = 1 - s->pb;
   } else {
-    if (branch) {
-      cudaEventRecord(s->ev_join, s->side);
-      cudaStreamWaitEvent(s->stream, s->ev_join, 0);
-    }
+    if (diag_branch) join();
     k_advance<<<1, 1, 0, s->stream>>>(s->dstate, s->cur);
   }
   s->cur = 1 - s->cur;

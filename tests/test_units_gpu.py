@@ -532,3 +532,32 @@ def test_staged_threshold_launches_no_sparse_kernel(M, tmp_path):  # noqa: F811
     for below, there in ((0, False), (1, False), (2, True), (1 << 30, True)):
         names = kernels_of_a_step(M, g, P, "P32", tmp_path / str(below), push_sparse_below=below)
         assert "k_push_tiled" in names and ("k_push_sparse" in names) == there, below
+
+
+@pytest.mark.parametrize("prec", ["P32", "P64"])
+def test_timed_steps_with_sparse_tiles(M, prec):  # noqa: F811
+    # the particle step's timed scope holds both its kernels side by side:
+    # timed steps, with power and bunch records, leave what untimed ones do
+    g = dict(inputs.random_grid(231, 40, 40, 48), boundary=1)
+    P = dict(inputs.random_particles(232, g, 30000, u_scale=0.3), q_macro=-1e-17)
+    tol = 1e-11 if prec == "P64" else 1e-5
+    recs = []
+    with M.Simulation(g, None, P, precision=getattr(M, prec)) as a, \
+            M.Simulation(g, None, P, precision=getattr(M, prec)) as b:
+        for s in (a, b):
+            s.set_tuning(push_sparse_below=100)
+            s.set_power_sampling(40, 20)
+            s.set_bunch_sampling(1.0e3, 1, 20)
+        a.profile(True)
+        a.step(9)
+        kt = a.kernel_times()
+        assert kt["push"][1] == 9 and kt["push"][0] > 0.0
+        b.step(9)
+        for s in (a, b):
+            recs.append((s.read_power(), s.read_bunch()))
+        for x, y in zip(*recs):
+            assert x.shape == y.shape and len(x) == 9
+            assert (np.abs(x - y) <= tol * np.abs(y).max(0) + 1e-30).all()
+        pa, pb = a.copy_particles(), b.copy_particles()
+        for nm in ("x", "uz"):
+            assert np.abs(pa[nm] - pb[nm]).max() <= tol * np.abs(pb[nm]).max()
