@@ -404,10 +404,11 @@ mithra_status mithra_read_spectrum(mithra_sim* sim, double* dW_domega, int64_t* 
  *   push_sparse_below: push variant 1 only; a tile holding fewer particles
  *     than this skips the shared-memory staging: one warp pushes its
  *     particles with E and B from global memory and deposits with global
- *     atomics, beside the CTAs that take the denser tiles (0: 32, FP64 64, on
- *     grids of at least 16 tiles per persistent CTA, and every tile staged on
- *     smaller ones; 1: every tile staged).  Takes effect from the tile list of
- *     the next re-sort.
+ *     atomics, beside the CTAs that take the denser tiles (0: 32 on grids of
+ *     at least 16 tiles per persistent CTA, in FP64 32 from 40 and 64 from 96
+ *     tiles on, or 64 from 28 on where the particles are 100 a tile, and every
+ *     tile staged on smaller ones; 1: every tile staged).  Takes effect from
+ *     the tile list of the next re-sort.
  * Defaults: stencil_variant 2 with lz 0 (the fastest form of the potential
  * update on every grid timed), push_variant 1 when the driver provides TMA
  * tensor maps (else 0), push_ctas_per_sm 0, push_sparse_below 0.

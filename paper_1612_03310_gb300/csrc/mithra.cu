@@ -513,18 +513,31 @@ int ring_run(const mithra_sim* s) {
 bool mur_all(const mithra_sim* s) { return s->g.boundary == 1 && xhi_fused(s->g.nx); }
 
 // Tiles below this many particles take the sparse path (0: none): the
-// caller's threshold, or 32 (FP64: 64) on grids of many tiles per CTA, where
-// the staged path's time is its number of tiles (128 x 128 x 1024 cells, 2^21
-// particles, P32_U64: 252 us at 0, 240 at 16 to 32, 273 at 64; FP64 on 96 x 80
-// x 384 cells, 4e5 particles: 536, 471 at 32, 458 at 64).  With few tiles a
-// CTA the lone warp of a sparse tile takes longer than a CTA with it, also in
-// a batch of many small members (64 of 32 x 32 x 128 cells and 2000
-// particles: 225 us a step staged, 238 at 32, 268 at 128).
+// caller's threshold, or the library's on grids of many tiles per persistent
+// CTA, where the staged path's time is its number of tiles (128 x 128 x 1024
+// cells, 2^21 particles, P32_U64, particle step: 252 us at 0, 240 at 16 to 32,
+// 273 at 64).  With few tiles a CTA the lone warp of a sparse tile takes
+// longer than a CTA with it, also in a batch of many small members (64 of 32 x
+// 32 x 128 cells and 2000 particles: 225 us a step staged, 238 at 32, 268 at
+// 128).  Where the lines lie, by the step with every tile staged and with the
+// threshold, of a Gaussian bunch:
+//   FP32 (three CTAs an SM), threshold 32, of 16 and of 64 particles a column:
+//   at 8 tiles a CTA 57.0 and 59.2 us, 95.4 and 99.6; at 12 73.2 and 71.1,
+//   106.7 and 104.9; at 16 84.3 and 80.1, 118.1 and 114.4;
+//   FP64 (one CTA an SM, whose registers leave a sparse block no room beside
+//   it), staged, 32 and 64.  Below 100 particles a tile of the grid on
+//   average: at 16 tiles a CTA 291, 351 and 369, at 38 571, 630 and 651, at 45
+//   698, 702 and 721 and (more particles) 850, 833 and 855, at 61 894, 876 and
+//   897, at 81 1165, 1122 and 1137, at 108 1485, 1410 and 1411.  Above: at 16
+//   583, 585 and 596, at 31 802, 811 and 795, at 38 1521, 1522 and 1502, at 61
+//   1629, 1587 and 1564, at 108 2760, 2697 and 2667.
 int sparse_below(const mithra_sim* s) {
   if (s->push_variant != 1 || !s->have_tm) return 0;
   if (s->push_sparse_below > 0) return s->push_sparse_below > 1 ? s->push_sparse_below : 0;
-  if (s->nkeys < 16 * s->push_grid) return 0;
-  return s->prec == MITHRA_P64 ? 64 : 32;
+  const int64_t tiles = s->nkeys, ctas = s->push_grid;
+  if (s->prec != MITHRA_P64) return tiles < 16 * ctas ? 0 : 32;
+  if (s->np >= 100 * tiles) return tiles < 28 * ctas ? 0 : 64;
+  return tiles < 40 * ctas ? 0 : tiles < 96 * ctas ? 32 : 64;
 }
 
 // Blocks of the sparse tiles' kernel: eight a multiprocessor (32 warps), so

@@ -503,26 +503,27 @@ def test_fused_batch_of_sparse_and_dense_members(M, prec):  # noqa: F811
             s.close()
 
 
-@pytest.mark.parametrize("prec,shape", [
-    ("P64", (64, 64, 304)), ("P64", (64, 64, 296)),
-    ("P32_U64", (128, 128, 232)), ("P32_U64", (128, 128, 224))])
-def test_automatic_sparse_threshold(M, orc, prec, shape, tmp_path):  # noqa: F811
-    # both sides of 16 tiles per persistent CTA (one a multiprocessor in FP64,
-    # three in FP32): sparse tiles in their own kernel, or every tile staged
-    per_sm = 1 if prec == "P64" else 3
+@pytest.mark.parametrize("prec,shape,per_tile,there", [
+    ("P64", (64, 128, 384), 40, True), ("P64", (64, 128, 376), 40, False),
+    ("P64", (64, 128, 272), 100, True), ("P64", (64, 128, 272), 99, False),
+    ("P64", (64, 128, 264), 100, False), ("P32_U64", (128, 128, 232), 40, True),
+    ("P32_U64", (128, 128, 224), 40, False)])
+def test_automatic_sparse_threshold(M, orc, prec, shape, per_tile, there, tmp_path):  # noqa: F811
+    # both sides of the lines: in FP64 (one persistent CTA a multiprocessor) 40
+    # tiles a CTA, or 28 with 100 particles a tile, in FP32 (three) 16; the
+    # sparse tiles in their own kernel, or every tile staged
     torch = pytest.importorskip("torch")
     n_sm = torch.cuda.get_device_properties(0).multi_processor_count
     tiles = shape[0] * shape[1] * shape[2] // 512
     if n_sm != 152:
-        pytest.skip("shapes are chosen for 152 multiprocessors")
+        pytest.skip("the shapes are chosen for 152 multiprocessors")
     g = dict(inputs.random_grid(211, *shape), boundary=1)
-    # 40 particles a tile on average: sparse and dense tiles under 32, sparse
-    # ones under 64 with a clump that is dense
-    P = inputs.random_particles(212, g, 40 * tiles, u_scale=0.2)
-    for a in "xyz":
-        P[a][:500] = P[a][0] + g["d" + a] * np.random.default_rng(213).random(500)
+    # four fifths of the particles in the lower half: sparse and dense tiles
+    P = dict(inputs.random_particles(212, g, per_tile * tiles, u_scale=0.2), q_macro=-1e-16)
+    far = np.random.default_rng(213).random(len(P["z"])) < 0.6
+    P["z"] = np.where(far & (P["z"] > g["nz"] / 2 * g["dz"]), P["z"] - (g["nz"] / 2 - 2) * g["dz"], P["z"])
     names = kernels_of_a_step(M, g, P, prec, tmp_path / "step")
-    assert ("k_push_sparse" in names) == (tiles >= 16 * per_sm * n_sm)
+    assert ("k_push_sparse" in names) == there
     check(M, orc, g, None, P, prec, (1, 3))
 
 
