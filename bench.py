@@ -144,21 +144,35 @@ class ClockSampler:
                 "samples": len(self.rows), "reasons": sorted(reasons)}
 
 
-# kernels behind one timed scope of the library's profiler: the potential
-# update is the Mur boundary kernel plus the interior kernel, the re-sort scan
-# two passes, the particle step the dense and the sparse tiles.  A smaller grid
-# takes as little as one kernel for the whole re-sort, one for every tile and
-# one for the update with its boundary.
-KERNELS_PER_SCOPE = {"potential_step": 2, "scan_counts": 2, "push": 2}
-SMALL_GRID_KEYS = 16 * 3 * 152  # tiles, 16 per persistent CTA
+N_SM = 152  # multiprocessors of a GB300
 
 
-def kernels_of(scope: str, n: int, grid: dict) -> int:
-    """Kernels launched by n occurrences of a timed scope, at least."""
-    keys = ((grid["nx"] + 7) // 8) * ((grid["ny"] + 7) // 8) * ((grid["nz"] + 7) // 8)
-    if keys > SMALL_GRID_KEYS:
-        return n * KERNELS_PER_SCOPE.get(scope, 1)
-    return 0 if scope == "slot_map" else n
+def kernels_of(scope: str, n: int, grid: dict, n_part: int, precision: str, tuning: dict) -> int:
+    """Kernels launched by n occurrences of a timed scope: the potential
+    update is the boundary kernel and the interior kernel, or one where the
+    register form does its whole boundary; the particle step the dense and
+    (with a threshold) the sparse tiles; the re-sort's scan two passes, or
+    with the slot map one kernel below 4096 tiles."""
+    nx, ny, nz = grid["nx"], grid["ny"], grid["nz"]
+    tiles = ((nx + 7) // 8) * ((ny + 7) // 8) * ((nz + 7) // 8)
+    p64 = precision == "p64"
+    if scope == "slot_map":
+        return n if tiles >= 4096 else 0
+    if scope == "scan_counts":
+        return 2 * n if tiles >= 4096 else n
+    if scope == "push":
+        below = tuning["push_sparse_below"]
+        if below == 0:  # the library's rule
+            ctas = N_SM * min(tuning["push_ctas_per_sm"] or 3, 1 if p64 else 3)
+            least = 16 if not p64 else 28 if n_part >= 100 * tiles else 40
+            below = 32 if tiles >= least * ctas else 1
+        return 2 * n if tuning["push_variant"] == 1 and below > 1 else n
+    if scope == "potential_step":
+        cols, rows = (nx + 31) // 32, (ny + 7) // 8
+        ring = (not p64 and cols * rows * nz >= 16 * N_SM and
+                10 * nx * ny >= 7 * 32 * cols * 8 * rows)
+        return n if tuning["stencil_variant"] == 2 and not ring and (nx - 1) % 32 else 2 * n
+    return n
 
 
 PRECISIONS = {"p32": "P32", "p32_u64": "P32_U64", "p32_c": "P32_C", "p64": "P64"}
@@ -358,7 +372,8 @@ def run_gpu(args, rank, world):
                                       for t in rec.get("trials", [])],
                grid=g, n_lost=parts["n_lost"], power_last=float(power[-1, 0]),
                source_reads=src_reads,
-               launches=sum(kernels_of(k, n, g) for k, (_, n) in kt.items()))
+               launches=sum(kernels_of(k, n, g, n_part, args.precision, tuning)
+                            for k, (_, n) in kt.items()))
 
     # the other precision forms on the same workload, shorter: P64 (plain
     # FP64) and P32_U64 (compensated FP32 levels, FP64 momenta: the form that

@@ -4,6 +4,7 @@ where they can go wrong: tiles of exactly one, a whole number and one more
 than a whole number of units, key counts around the scans' block sizes, the
 sparse tiles' kernel beside the units, an empty bunch; against the oracle."""
 import ctypes as C
+import re
 from concurrent.futures import ThreadPoolExecutor
 
 import numpy as np
@@ -562,3 +563,26 @@ def test_timed_steps_with_sparse_tiles(M, prec):  # noqa: F811
         pa, pb = a.copy_particles(), b.copy_particles()
         for nm in ("x", "uz"):
             assert np.abs(pa[nm] - pb[nm]).max() <= tol * np.abs(pb[nm]).max()
+
+
+@pytest.mark.parametrize("prec", ["P32", "P32_U64", "P64"])
+@pytest.mark.parametrize("shape,n,tuning", [
+    ((32, 32, 64), 500, {}), ((33, 32, 64), 500, {}), ((64, 64, 320), 2000, {}),
+    ((65, 65, 256), 0, {}), ((128, 64, 264), 2000, dict(push_sparse_below=16)),
+    ((64, 128, 280), 250000, {}), ((64, 128, 400), 2000, {}), ((128, 128, 240), 2000, {}),
+    ((128, 128, 240), 2000, dict(push_ctas_per_sm=1, stencil_variant=0)),
+    ((48, 48, 48), 500, dict(push_variant=0))])
+def test_kernels_that_the_bench_counts(M, prec, shape, n, tuning, tmp_path):  # noqa: F811
+    # bench.kernels_of against the kernels of a captured step: each form of the
+    # update, of the particle step and of the re-sort
+    from test_replicas_cpu import _bench
+    g = dict(inputs.random_grid(241, *shape), boundary=1)
+    P = inputs.random_particles(242, g, n, u_scale=0.2) if n else None
+    names = kernels_of_a_step(M, g, P, prec, tmp_path / "step", **tuning)
+    full = dict(stencil_variant=2, lz=0, push_variant=1, push_ctas_per_sm=0, push_sparse_below=0)
+    full.update(tuning)
+    scopes = ["potential_step"] + (["push", "scan_counts", "slot_map"] if n else [])
+    count = sum(_bench().kernels_of(k, 1, g, n, prec.lower(), full) for k in scopes)
+    found = re.findall(r"6mithra\d+(k_[a-z_0-9]+?)(?=[IE])", names)
+    # (without particles, the kernel that advances the step counter)
+    assert len(found) == count + (0 if n else 1), (count, found)
