@@ -289,7 +289,12 @@ const char* mithra_last_error(const mithra_sim* sim);
  * for the stream and returns, per kernel id k < *n_kernels, the summed
  * duration ms[k] (milliseconds) and the number of launches[k] since
  * profiling was enabled (arrays of max_kernels entries).  mithra_kernel_name
- * names kernel id k (NULL when out of range). */
+ * names kernel id k (NULL when out of range).  A scope holds all the kernels of
+ * its part of the step: the potential update with its boundary, the particle
+ * step's dense and sparse tiles (beside each other, as in an untimed step),
+ * both passes of the scan.  Where the re-sort is one kernel (at most 4095
+ * tiles) its time is scan_counts', and slot_map's event pairs hold nothing
+ * between them. */
 mithra_status mithra_profile(mithra_sim* sim, int32_t enable);
 mithra_status mithra_kernel_times(mithra_sim* sim, double* ms, int64_t* launches,
                                   int32_t max_kernels, int32_t* n_kernels);

@@ -79,8 +79,9 @@ struct ZParams {
 template <bool kLo, typename T>
 __global__ void __launch_bounds__(256) kb_mur(const __grid_constant__ ZParams<T> prm) {
   // placed while the re-sort drains, and kb_potential as the last blocks here
-  // run (step of 64 members of 32 x 32 x 128 cells: 158.6 to 155.3 us, P32_U64
-  // 209.6 to 206.5; of 200 members 445 to 439)
+  // run (step of 64 members of 32 x 32 x 128 cells with 2000 particles in 36
+  // tiles each: 158.6 to 155.3 us, P32_U64 209.6 to 206.5; of 200 members 445
+  // to 439)
   grid_dep_wait();
   grid_dep_launch();
   const int g = blockIdx.x;

@@ -509,7 +509,8 @@ int ring_run(const mithra_sim* s) {
 // kernel and without: 32 x 32 x 64 cells 11.5 and 8.1 us, in FP64 37 and 23;
 // 96 x 80 x 384 in FP64 483 and 451), unless the x+ face's lanes cannot share
 // a warp with their neighbours.  A fused batch keeps the boundary kernel (64
-// members of 32 x 32 x 128 cells: 212 us a step with it, 217 without).
+// members of 32 x 32 x 128 cells with 2000 particles in 46 tiles each: 212 us
+// a step with it, 217 without; 204 since, with its launches overlapped).
 bool mur_all(const mithra_sim* s) { return s->g.boundary == 1 && xhi_fused(s->g.nx); }
 
 // Tiles below this many particles take the sparse path (0: none): the
@@ -2370,7 +2371,8 @@ mithra_status capture_fused_typed(mithra_batch* b) {
     // sparse tiles and the particle step of each group of up to kPushGroup
     // members (their arguments in the launch's parameter space) beside each
     // other: one group alone leaves the device partly idle (64 members of 32 x
-    // 32 x 128 cells, 2000 particles: three groups one after another 86 us)
+    // 32 x 128 cells, 2000 particles in 46 tiles each: three groups one after
+    // another 86 us)
     auto fork = [&](int r) {
       cudaEventRecord(b->ev_branch[r], q);
       cudaStreamWaitEvent(b->branch[r], b->ev_branch[r], 0);

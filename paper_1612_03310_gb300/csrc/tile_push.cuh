@@ -381,8 +381,11 @@ __global__ void __launch_bounds__(kPushThreads, (sizeof(T) == 4 ? 3 : 1))
   // list's entry) do not stand between two units: under the charge block's
   // flush, or, for units of one round of particles in a list of many per CTA,
   // under the boxes' flight and the E/B phase (taken that early, the last
-  // units wait for CTAs still at work: c2, 7 units a CTA, 240 -> 248 us; 64
-  // batch members of 2000 particles, 14 a CTA, 225 -> 210 us a step).
+  // units wait for CTAs still at work).  Step with every unit claimed late and
+  // early, tiles of 60 and of 200 particles: 4 units a CTA 50.3 and 50.4 us,
+  // 61.7 and 62.6; 8 106.5 and 104.7, 132.0 and 131.7; 10 126.1 and 123.4,
+  // 153.2 and 152.0; 14 175.0 and 171.3, 212.3 and 211.6; a bunch's tiles of
+  // 165 to 620 at 2 a CTA 169.2 and 170.3, 199.3 and 202.4.
   constexpr int kClaim = kPushThreads - 32;
   const bool many = units() >= 10 * (int)gridDim.x;
   auto dense = [&](const PushArgs<T, U>& a, const CUtensorMap* tmp, const CUtensorMap* tmd,
