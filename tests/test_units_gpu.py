@@ -586,3 +586,23 @@ def test_kernels_that_the_bench_counts(M, prec, shape, n, tuning, tmp_path):  # 
     found = re.findall(r"6mithra\d+(k_[a-z_0-9]+?)(?=[IE])", names)
     # (without particles, the kernel that advances the step counter)
     assert len(found) == count + (0 if n else 1), (count, found)
+
+
+@pytest.mark.parametrize("prec,nx", [("P32", 64), ("P32_C", 64), ("P32_C", 67)])
+def test_ring_runs_agree(M, prec, nx):  # noqa: F811
+    # runs from one plane (fewer planes than stages) to more than the grid has:
+    # the same arithmetic whatever the run, to the bit
+    g = dict(inputs.random_grid(251, nx, 62, 275), boundary=1)
+    f = smooth_levels(g)
+    n = nx * 62 * 275
+    out = {}
+    for lz in (0, 1, 2, 3, 16, 300):
+        with M.Simulation(g, None, None, precision=getattr(M, prec)) as sim:
+            sim.set_tuning(lz=lz)
+            for a, nm in enumerate(("Ax", "Ay", "Az", "phi")):
+                sim.set_field(nm + "_prev", f["prev"][a * n:(a + 1) * n])
+                sim.set_field(nm, f["cur"][a * n:(a + 1) * n])
+            sim.step(5)
+            out[lz] = [sim.copy_field(nm) for nm in ("Ax", "phi", "Az_prev")]
+    for lz, fields in out.items():
+        assert all(np.array_equal(a, b) for a, b in zip(fields, out[0])), lz
